@@ -67,13 +67,6 @@ WORKLOADS = {
                   "fraction 0.42 over the box)"),
 }
 HBM_FALLBACK_GBS = 6800.0
-# FP64 arithmetic peak of the GPU: 2 FP64 fused multiply-adds per clock per SM
-FP64_FMA_PER_CLK_SM = 2
-# algorithmic FP64 flops of the collision (adds and multiplies, a fused
-# multiply-add counts 2): per cell (moments, equilibrium, TRT relaxation with
-# forcing, (1 - B) weighting) and per occupied slot (solid operator and force)
-FLOP_PER_CELL = 219
-FLOP_PER_SLOT = 139
 
 
 def peaks():
@@ -170,10 +163,6 @@ class ClockSampler:
 def source_hash(path):
     with open(path, "rb") as f:
         return hashlib.sha256(f.read()).hexdigest()[:16]
-
-
-def fp64_peak_tflops(sm_max_mhz, sm_count):
-    return sm_count * FP64_FMA_PER_CLK_SM * 2 * sm_max_mhz * 1e6 / 1e12
 
 
 def profiled_traffic(kernel_src, name, cells):
@@ -352,18 +341,13 @@ def train_surrogate(capi, seed=20230321):
                     "seconds": time.perf_counter() - t0}
 
 
-def collide_roofline(prec, cells, ncov, nslot, coll_ms, hbm, sm_count):
-    if prec != "fp64":
-        b = (152 * cells + 16 * ncov) if prec == "fp32" else (304 * cells + 24 * ncov)
-        gbs = b / (coll_ms * 1e-3) / 1e9
-        return {"collide_hbm_gbs": gbs, "collide_hbm_frac": gbs / hbm}
-    tf = (FLOP_PER_CELL * cells + FLOP_PER_SLOT * nslot) / (coll_ms * 1e-3) / 1e12
-    return {"collide_fp64_tflops": tf,
-            "collide_fp64_frac": tf / fp64_peak_tflops(2070.0, sm_count),
-            "collide_hbm_frac": (304 * cells + 24 * ncov) / (coll_ms * 1e-3) / 1e9 / hbm}
+def collide_roofline(prec, cells, ncov, coll_ms, hbm):
+    b = (152 * cells + 16 * ncov) if prec == "fp32" else (304 * cells + 24 * ncov)
+    gbs = b / (coll_ms * 1e-3) / 1e9
+    return {"collide_hbm_gbs": gbs, "collide_hbm_frac": gbs / hbm}
 
 
-def forms_comparison(capi, torch, params, sm_count, steps=CHANNEL_STEPS):
+def forms_comparison(capi, torch, params, steps=CHANNEL_STEPS):
     """The metric's second half on the channel workload (256x256x512, walls at
     the x faces, 12,817 fixed spheres r=5, TRT tau=0.55, body force 1e-5 along
     z), over the 5,000 steps the workload is defined for: FP64 PDFs with 8^3
@@ -402,14 +386,13 @@ def forms_comparison(capi, torch, params, sm_count, steps=CHANNEL_STEPS):
         t = e.timings()
         e.set_timing(False)
         coll_ms = t[1] / t[4]
-        p0, _, p1, _ = e.slots()
+        p0, _, _, _ = e.slots()
         ncov = int((p0 >= 0).sum())
-        nslot = ncov + int((p1 >= 0).sum())
         F, _ = e.force_torque()
         _, u = e.macroscopic()
         r = {"mlups": w.cells * (steps - 11) / (ms * 1e-3) / 1e6, "mapping_ms_once": map_ms,
              "collide_ms": coll_ms}
-        r.update(collide_roofline(prec, w.cells, ncov, nslot, coll_ms, hbm, sm_count))
+        r.update(collide_roofline(prec, w.cells, ncov, coll_ms, hbm))
         res[name] = (r, F, u)
         e.close()
         torch.cuda.empty_cache()
@@ -441,7 +424,7 @@ def settling_summary(w, e, mass):
             "mean_drag_z": float(np.mean(F[:, 2]))}
 
 
-def forms_settling(capi, torch, params, ref, steps, sm_count):
+def forms_settling(capi, torch, params, ref, steps):
     """The moving-particle form of the metric on the 512x512x1024 periodic box
     (268M cells, 94,692 spheres r in [3, 6] at solid fraction 0.15, density
     ratio 2.5, gravity, DEM).  `ref` is the plain FP64 method (8^3 sampling,
@@ -473,13 +456,12 @@ def forms_settling(capi, torch, params, ref, steps, sm_count):
         e.step(3)
         t = e.timings()
         e.set_timing(False)
-        p0, _, p1, _ = e.slots()
+        p0, _, _, _ = e.slots()
         ncov = int((p0 >= 0).sum())
-        nslot = ncov + int((p1 >= 0).sum())
         r = {"mlups": w.cells * k / (ms * 1e-3) / 1e6, "ms_per_step": ms / k,
              "mapping_ms_per_step": t[0] / t[4], "collide_ms": t[1] / t[4],
              "force_ms": t[2] / t[4], "dem_ms": t[3] / t[4]}
-        r.update(collide_roofline(prec, w.cells, ncov, nslot, r["collide_ms"], hbm, sm_count))
+        r.update(collide_roofline(prec, w.cells, ncov, r["collide_ms"], hbm))
         r.update(settling_summary(w, e, mass))
         r["speedup_vs_fp64"] = r["mlups"] / ref["mlups"]
         r["settling_velocity_rel_diff"] = abs(r["mean_settling_velocity"] /
@@ -565,7 +547,6 @@ def main():
 
     import torch
     torch.cuda.set_device(local)
-    sm_count = torch.cuda.get_device_properties(local).multi_processor_count
     dist = None
     if world > 1:
         import torch.distributed as dist
@@ -626,8 +607,9 @@ def main():
     bytes_psm = bytes_lbm + ncov * (24 if esz == 8 else 16)
     hbm, peak_kind = peaks()
     hbm_achieved = bytes_psm / (lbm_ms * 1e-3) / 1e9
-    # the collision kernel of the form: FP64 on compacted warps, FP32 AA
-    # staged, FP32 pull and double-float one cell per thread
+    # the collision kernel of the form: FP64 in fixed point, the cells without
+    # particles staged and (timed with it) the covered cells; FP32 AA staged;
+    # FP32 pull and double-float one cell per thread
     if fp64:
         kbase, kname = "lbm_fp64_kernel", f"lbm_fp64_kernel<{args.streaming}>"
     else:
@@ -637,29 +619,14 @@ def main():
     traffic = profiled_traffic(os.path.join(ROOT, "paper_2303_11811_gb300", "csrc",
                                             "lbm_kernels.cu"),
                                f"{kbase}_{args.precision}{args.streaming}_{args.workload}", cells)
-    hbm_part = {"achieved": hbm_achieved, "peak": hbm, "unit": "GB/s",
-                "frac": hbm_achieved / hbm, "peak_source": peak_kind,
-                "bytes_per_launch": bytes_psm, "lbm_only_bytes_per_launch": bytes_lbm}
     common = {"kernel": kname, "traffic": traffic, "covered_cells": ncov, "slots": nslot,
               "avg_launch_ms": lbm_ms,
               "class_ms_per_step": {"mapping": t[0] / t[4], "stream_collide": lbm_ms,
                                     "force_reduce": t[2] / t[4], "dem": t[3] / t[4]}}
-    if fp64:
-        # FP64 runs at 1/64 of the FP32 rate on this GPU: the FP64 pipe binds
-        sm_max = (clk or {}).get("sm_max_mhz") or 2070.0
-        peak = fp64_peak_tflops(sm_max, sm_count)
-        flops = FLOP_PER_CELL * cells + FLOP_PER_SLOT * nslot
-        achieved = flops / (lbm_ms * 1e-3) / 1e12
-        roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                    "frac": achieved / peak,
-                    "peak_source": f"derived: {sm_count} SMs x {FP64_FMA_PER_CLK_SM} FP64 "
-                                   f"FMA/clk x 2 flop x {sm_max:.0f} MHz",
-                    "flops_per_launch": flops, "hbm": hbm_part, **common}
-    else:
-        roofline = {"bound": "hbm", "achieved": hbm_achieved, "peak": hbm, "unit": "GB/s",
-                    "frac": hbm_achieved / hbm, "peak_source": peak_kind,
-                    "bytes_per_launch": bytes_psm, "lbm_only_bytes_per_launch": bytes_lbm,
-                    **common}
+    roofline = {"bound": "hbm", "achieved": hbm_achieved, "peak": hbm, "unit": "GB/s",
+                "frac": hbm_achieved / hbm, "peak_source": peak_kind,
+                "bytes_per_launch": bytes_psm, "lbm_only_bytes_per_launch": bytes_lbm,
+                **common}
 
     # end to end through the C ABI with host buffers in pinned memory
     n = w.particles["r"].size
@@ -716,14 +683,14 @@ def main():
         ref = {"mlups": value, "ms_per_step": ms / args.steps,
                "mapping_ms_per_step": t[0] / t[4], "collide_ms": lbm_ms,
                "force_ms": t[2] / t[4], "dem_ms": t[3] / t[4]}
-        ref.update(collide_roofline("fp64", cells, ncov, nslot, lbm_ms, hbm, sm_count))
+        ref.update(collide_roofline("fp64", cells, ncov, lbm_ms, hbm))
         ref.update(settling_summary(w, e, mass))
     e.close()
     torch.cuda.empty_cache()
     if default_run and not args.no_forms and rank == 0:
         forms = {"surrogate_training": training,
-                 "settling": forms_settling(capi, torch, params, ref, settle_steps, sm_count),
-                 "channel": forms_comparison(capi, torch, params, sm_count)}
+                 "settling": forms_settling(capi, torch, params, ref, settle_steps),
+                 "channel": forms_comparison(capi, torch, params)}
 
     cpu = None
     if rank == 0 and world == 1 and not args.no_cpu_baseline and w.eps_mode != "mlp":

@@ -20,12 +20,8 @@
 namespace psm {
 namespace {
 
-// element traits: FP64 (the warp-shared solid operator, FP64-pipe bound), or
-// a form that runs on the FP32 pipes (FP32 deviations, double-float pairs)
-template <typename T>
-constexpr bool kFP64 = false;
-template <>
-constexpr bool kFP64<double> = true;
+// element traits: the double-float form runs on the FP32 pipes like FP32; the
+// FP64 form has kernels of its own below
 template <typename T>
 constexpr bool kDF = false;
 template <>
@@ -186,27 +182,7 @@ __device__ __forceinline__ const CollideCoef<df>* coef_of<df>(const StepConst* s
   return &sc->x;
 }
 
-// Shared memory of one warp for the FP64 solid operator.  Work is split in
-// "jobs" (one per covered cell and occupied slot) and "items" (job x
-// direction pair, 9 per job) spread over all 32 lanes, so that the FP64 work
-// of a warp with a few covered cells is not repeated by its idle lanes.  The
-// items add their results to a shared copy of the owner lane's PDFs, slot 0
-// before slot 1.
-template <typename T>
-struct SolidSmem {
-  T cu[32][9];     // per lane: c_k . U_f of its cell
-  T am[32][9];     // per lane: antisymmetric moments a_k of its cell
-  T dd[32][18];    // per lane: its PDFs 1..18 while the items add to them
-  T cv[32][9];     // per job: c_k . U_p
-  T con[32][7];    // per job: alpha, beta, gamma for faces and edges, B_i
-  int owner[32];
-};
 constexpr int LBM_THREADS = 256;
-
-template <typename T>
-size_t lbm_smem_bytes() {
-  return sizeof(SolidSmem<T>) * (LBM_THREADS / 32);
-}
 
 // Force of one slot on its particle (Eq. 21): B_i sum_q C^s_q c_qbar =
 // -2 B_i sum_k A_k c_k over the pairs, with A_k = 3 w_k c_k.(U_f + U_p) - a_k.
@@ -250,13 +226,12 @@ __device__ __forceinline__ void load_slot_rec(const LbmParams& P, uint32_t m, in
 
 // Collision of one cell (Eqs. 3-8 and 17-21) on the PDFs d gathered by the
 // streaming step; the warp's 32 lanes hold the 32 cells of coverage word
-// `word` (padding lanes compute on a copy of a real cell).  FP64 kernels
-// pass the warp's SolidSmem.
+// `word` (padding lanes compute on a copy of a real cell).
 // `pre` holds the cell's slot record when the kernel loaded it ahead (PRE),
 // else the record is read here.
 template <typename T, bool PRE>
 __device__ __forceinline__ void psm_collide(const LbmParams& P, unsigned word, int lane, bool live,
-                                            T* d, SolidSmem<T>* solid, uint32_t m, int eb,
+                                            T* d, uint32_t m, int eb,
                                             const SlotRec<T>* pre) {
   // ---- the cell's slots; the second one's record is read only when present
   bool cov, has1 = false;
@@ -344,10 +319,7 @@ __device__ __forceinline__ void psm_collide(const LbmParams& P, unsigned word, i
     }
   }
 
-  // ---- solid operator of each overlapping particle (Eqs. 19-21).  In FP64
-  // (1/64 of the FP32 rate here) the work is shared out over the lanes of the
-  // warp; in FP32 each covered lane does its own cell.
-  if constexpr (!kFP64<T>) {
+  // ---- solid operator of each overlapping particle (Eqs. 19-21)
   if (cov) {
 #pragma unroll 1
     for (int sl = 0; sl < 2; ++sl) {
@@ -368,71 +340,6 @@ __device__ __forceinline__ void psm_collide(const LbmParams& P, unsigned word, i
         d[2 * k + 2] += BdS - BA;
       }
       slot_force<T>(P, e, sl, Bi, Ux - Vx, Uy - Vy, Uz - Vz, h + CC_F);
-    }
-  }
-  } else if (m != 0u) {
-    SolidSmem<T>& S = *solid;
-    const bool has0 = cov, hs1 = cov && has1;
-    const unsigned b0 = __ballot_sync(0xffffffffu, has0);
-    const unsigned b1 = __ballot_sync(0xffffffffu, hs1);
-    const unsigned below = (1u << lane) - 1u;
-    if (has0) {
-#pragma unroll
-      for (int k = 0; k < 9; ++k) {
-        S.cu[lane][k] = cdot<T>(k, Ux, Uy, Uz);
-        S.am[lane][k] = a[k];
-      }
-#pragma unroll
-      for (int q = 1; q < Q; ++q) S.dd[lane][q - 1] = d[q];
-    }
-    // the jobs of slot 0, then those of slot 1: within a pass each owner lane
-    // has at most one job, so no two items of a pass update the same PDF
-#pragma unroll
-    for (int sl = 0; sl < 2; ++sl) {
-      const unsigned bs = sl ? b1 : b0;
-      if (bs == 0u) continue;
-      const int Js = __popc(bs);
-      if (sl ? hs1 : has0) {
-        // job set-up by the owner lane: the per-job constants of the item
-        // arithmetic and the slot's force (Eq. 21)
-        const int jj = __popc(bs & below);
-        const T Vx = sl ? r1[0] : r0[0], Vy = sl ? r1[1] : r0[1], Vz = sl ? r1[2] : r0[2];
-        const T Bi = sl ? r1[3] : r0[3];
-        const T dU2 = (Vx * Vx + Vy * Vy + Vz * Vz) - uu;
-        d[0] += Bi * (T(-1.5) * w0<T>() * dU2);
-#pragma unroll
-        for (int k = 0; k < 9; ++k) S.cv[jj][k] = cdot<T>(k, Vx, Vy, Vz);
-        const T BdU = Bi * dU2;
-        S.con[jj][0] = (T(4.5) * wk<T>(0)) * Bi;
-        S.con[jj][1] = (T(-1.5) * wk<T>(0)) * BdU;
-        S.con[jj][2] = (T(3) * wk<T>(0)) * Bi;
-        S.con[jj][3] = (T(4.5) * wk<T>(3)) * Bi;
-        S.con[jj][4] = (T(-1.5) * wk<T>(3)) * BdU;
-        S.con[jj][5] = (T(3) * wk<T>(3)) * Bi;
-        S.con[jj][6] = Bi;
-        S.owner[jj] = lane;
-        slot_force<T>(P, e, sl, Bi, Ux - Vx, Uy - Vy, Uz - Vz, h + CC_F);
-      }
-      __syncwarp();
-      // items: job j, pair k, added to the owner's PDFs.  C^s has symmetric
-      // part B_i w_k (9/2 (cv^2 - cu^2) - 3/2 dU2) and antisymmetric part
-      // B_i (3 w_k (cu + cv) - a_k)
-      for (int t = lane; t < 9 * Js; t += 32) {
-        const int j = t / 9, k = t - 9 * j;
-        const int L = S.owner[j];
-        const T cu = S.cu[L][k], cv = S.cv[j][k];
-        const int cl = k < 3 ? 0 : 3;
-        const T Dv = cv - cu, Sv = cv + cu;
-        const T BdS = S.con[j][cl] * (Dv * Sv) + S.con[j][cl + 1];
-        const T BA = S.con[j][cl + 2] * Sv - S.con[j][6] * S.am[L][k];
-        S.dd[L][2 * k] += BdS + BA;
-        S.dd[L][2 * k + 1] += BdS - BA;
-      }
-      __syncwarp();
-    }
-    if (has0) {
-#pragma unroll
-      for (int q = 1; q < Q; ++q) d[q] = S.dd[lane][q - 1];
     }
   }
   if constexpr (kDF<T>) {
@@ -553,6 +460,24 @@ __device__ __forceinline__ void store_pdfs(const LbmParams& P, const NbrT<WALLS>
 #undef DST
 }
 
+// the store of one direction (store_pdfs), q known at compile time
+template <typename T, int MODE, int WALLS>
+__device__ __forceinline__ void store_pdf(const LbmParams& P, const NbrT<WALLS>& nb, int cell,
+                                          int q, T v) {
+  const int k = (q - 1) >> 1, sg = (q & 1) ? 1 : -1, qr = q + sg;
+  if (q == 0) {
+    static_cast<T*>(P.dstq[0])[cell] = v;
+  } else if (MODE == 0) {
+    static_cast<T*>(P.dstq[q])[cell] = v;
+  } else if (MODE == 1) {
+    static_cast<T*>(P.dstq[qr])[cell] = v;
+  } else {
+    const int cx = sg * ckx(k), cy = sg * cky(k), cz = sg * ckz(k);
+    if (nb.ok(cx, cy, cz)) static_cast<T*>(P.dstq[q])[nb.idx(cx, cy, cz)] = v;
+    else static_cast<T*>(P.dstq[qr])[cell] = v;
+  }
+}
+
 // components of c_q in the canonical ordering (q = 2k+1: +c_k, q = 2k+2: -c_k)
 __device__ __forceinline__ int qsign(int q) { return (q & 1) ? 1 : -1; }
 
@@ -586,12 +511,11 @@ __device__ __forceinline__ void prefetch_span(const LbmParams& P, unsigned bn, i
   prefetch_l2(static_cast<const T*>(P.srcq[q]) + c0, (unsigned)((c1 - c0) * sizeof(T)));
 }
 
-// FP32 kernels are bandwidth bound and want resident warps (4 blocks per
-// SM); FP64 kernels are FP64-pipe bound and keep their registers
+// FP32 kernels are bandwidth bound and want resident warps (4 blocks per SM);
+// the double-float form is bound by the FP32 pipes and keeps its registers
 template <typename T, int MODE, int WALLS>
-__global__ void __launch_bounds__(LBM_THREADS, kFP64<T> ? 1 : (sizeof(T) == 4 ? 4 : 2))
+__global__ void __launch_bounds__(LBM_THREADS, sizeof(T) == 4 ? 4 : 2)
     lbm_kernel(LbmParams P) {
-  extern __shared__ __align__(16) unsigned char lbm_smem[];
   const Grid& g = P.g;
   if constexpr (sizeof(T) == 4) {
     if (P.pf_ahead > 0 && threadIdx.x < Q && blockIdx.x + (unsigned)P.pf_ahead < gridDim.x)
@@ -643,9 +567,7 @@ __global__ void __launch_bounds__(LBM_THREADS, kFP64<T> ? 1 : (sizeof(T) == 4 ? 
 
   if constexpr (MODE == 0) apply_open_faces<T, WALLS>(P, nb, z, cell, d);
 #undef SRC
-  psm_collide<T, false>(P, warp, lane, live, d,
-                        reinterpret_cast<SolidSmem<T>*>(lbm_smem) + (threadIdx.x >> 5), m, eb,
-                        nullptr);
+  psm_collide<T, false>(P, warp, lane, live, d, m, eb, nullptr);
   if (live) store_pdfs<T, MODE, WALLS>(P, nb, cell, d);
 }
 
@@ -799,20 +721,16 @@ __global__ void __launch_bounds__(BULK_THREADS, sizeof(T) == 4 ? 2 : 1)
   }
 
   // ---- consumers
-  SolidSmem<T>* solid = reinterpret_cast<SolidSmem<T>*>(
-                            bulk_smem + BULK_BAR_BYTES + S * stage_elems * sizeof(T)) + warp;
 #define SRC(q) static_cast<const T*>(P.srcq[q])
-  // FP32: the coverage word and first slot of a word are loaded one word
-  // ahead (the slot records of the collision depend on them): the word a
-  // warp takes next is w + 8 in the same tile, else its first word in the
-  // block's next tile.  Word index of (tile, w): tile * TR * wpr + w.  FP64
-  // loads them at the word.
-  constexpr bool ahead = !kFP64<T>;
+  // the coverage word and first slot of a word are loaded one word ahead (the
+  // slot records of the collision depend on them): the word a warp takes next
+  // is w + 8 in the same tile, else its first word in the block's next tile.
+  // Word index of (tile, w): tile * TR * wpr + w.
   const int tile_words = TR * g.wpr;
   auto words_in = [&](int t) { return min(TR, nrows - t * TR) * g.wpr; };
   uint32_t m_next = 0u;
   int eb_next = 0;
-  if (ahead && P.mask && blockIdx.x < P.ntiles && warp < words_in(blockIdx.x)) {
+  if (P.mask && blockIdx.x < P.ntiles && warp < words_in(blockIdx.x)) {
     const unsigned w0 = (unsigned)(blockIdx.x * tile_words + warp);
     m_next = __ldg(&P.mask[w0]);
     eb_next = __ldg(&P.base[w0]);
@@ -835,13 +753,12 @@ __global__ void __launch_bounds__(BULK_THREADS, sizeof(T) == 4 ? 2 : 1)
       const int x = live ? xr : g.nx - 1;
       const int row = row0 + r;
       const unsigned word = (unsigned)(row * g.wpr + wr);
-      const uint32_t m = ahead ? m_next : (P.mask ? __ldg(&P.mask[word]) : 0u);
-      const int eb = ahead ? eb_next : (P.mask ? __ldg(&P.base[word]) : 0);
-      // FP32: the record loads go out before the PDF reads; FP64 (bound by
-      // its pipe, registers tight) reads them in the collision
+      const uint32_t m = m_next;
+      const int eb = eb_next;
+      // the record loads go out before the PDF reads
       SlotRec<T> R;
-      if constexpr (ahead) load_slot_rec<T>(P, m, eb, lane, live, R);
-      if (ahead && P.mask) {
+      load_slot_rec<T>(P, m, eb, lane, live, R);
+      if (P.mask) {
         int t2 = tile, w2 = w + BULK_CONSUMER_WARPS;
         if (w2 >= nw) {
           t2 = tile + gridDim.x;
@@ -880,7 +797,7 @@ __global__ void __launch_bounds__(BULK_THREADS, sizeof(T) == 4 ? 2 : 1)
         }
       }
       if constexpr (MODE == 0) apply_open_faces<T, WALLS>(P, nb, z, cell, d);
-      psm_collide<T, ahead>(P, word, lane, live, d, solid, m, eb, &R);
+      psm_collide<T, true>(P, word, lane, live, d, m, eb, &R);
       if (live) store_pdfs<T, MODE, WALLS>(P, nb, cell, d);
     }
     __syncwarp();
@@ -889,24 +806,18 @@ __global__ void __launch_bounds__(BULK_THREADS, sizeof(T) == 4 ? 2 : 1)
 #undef SRC
 }
 
-// ---- FP64 collision on compacted warps.  FP64 runs at 1/64 of the FP32
-// rate on GB300, so the FP64 kernel is bound by its count of FP64
-// instructions.  Two things cost instructions on warps of 32 consecutive
-// cells: a warp with a covered cell weights every lane's fluid change by
-// (1 - B), and the solid operator of a few covered lanes keeps the whole warp
-// busy.  So each tile's cells are listed in three groups (uncovered cells,
-// covered cells, covered cells of one particle with B = 1) and warps take 32
-// list entries at a time: a warp of uncovered cells runs the particle-free
-// form, a warp of full cells the solid operator alone, any other warp every
-// lane's own fluid change and solid operators; at most two warps per tile
-// are mixed.
+// ---- FP64 collision on compacted warps, for the cells that the fixed-point
+// form (fixed64.cuh) does not take: deviations or velocities of 1/8 and more,
+// NaN, cells of two particles.
 enum { CK_UNCOVERED = 0, CK_MIXED = 1, CK_FULL = 2 };
-
-// the step's FP64 collision coefficients sit in shared memory (copied once
-// per block): the same four values for every lane, read as two 16-byte
-// broadcasts, which keeps them off the L1/texture path of the slot records
-constexpr int F64_COEF_BYTES = 512;
-static_assert(sizeof(CollideCoef<double>) <= F64_COEF_BYTES, "coefficient area");
+// consumer warps of the staged kernel: with the copy and the list warp a
+// multiple of four, which is what registers are shared out by.  14 (128
+// registers, no spills) measured best: 741 clocks of an SM per warp of cells
+// with 10, 645 with 14, 18 (96 registers) no faster on boxes with particles
+constexpr int F64_CONSUMER_WARPS = 14;
+constexpr int F64_THREADS = 32 * (F64_CONSUMER_WARPS + 2);
+constexpr int F64_FX_BYTES = (int)((sizeof(FxRow) * FX_ROWS + 127) / 128 * 128);
+constexpr int F64_TICKET_BYTES = 128;
 __device__ __forceinline__ void lds4(const double* p, double* o) {
   const double2 u = reinterpret_cast<const double2*>(p)[0];
   const double2 v = reinterpret_cast<const double2*>(p)[1];
@@ -929,9 +840,22 @@ __device__ __forceinline__ void lds4(const double* p, double* o) {
 // its slots (Eq. 19); an uncovered lane has B = 0.
 // Covered lanes write their slots' forces (Eq. 21).
 
+struct F64Slots {
+  const double* V;  // Slots::V
+  double* Fc;       // Slots::Fc
+  long long cap;
+  __device__ __forceinline__ void force(int e, int sl, double Bi, double dux, double duy,
+                                        double duz, const double* f) const {
+    double* o = Fc + 3 * ((long long)sl * cap + e);
+    o[0] = Bi * (dux - f[0]);
+    o[1] = Bi * (duy - f[1]);
+    o[2] = Bi * (duz - f[2]);
+  }
+};
+// (out of line: the fixed-point form takes almost every warp)
 template <int KIND>
-__device__ __forceinline__ void fp64_collide(const LbmParams& P, const CollideCoef<double>* cf,
-                                             double* d, bool cov, int e) {
+__device__ __noinline__ void fp64_collide(const F64Slots P, const CollideCoef<double>* cf,
+                                          double* d, bool cov, int e) {
   using T = double;
   T a[9], sk[9];
 #pragma unroll
@@ -976,7 +900,7 @@ __device__ __forceinline__ void fp64_collide(const LbmParams& P, const CollideCo
     }
   } else if constexpr (KIND == CK_FULL) {
     T r0[4] = {T(0), T(0), T(0), T(0)};
-    if (cov) ld4(static_cast<const T*>(P.slot_V) + 4LL * e, r0);
+    if (cov) ld4(P.V + 4LL * e, r0);
     const T Vx = r0[0], Vy = r0[1], Vz = r0[2];
     const T dU2 = (Vx * Vx + Vy * Vy + Vz * Vz) - uu;
     d[0] += (T(-1.5) * w0<T>()) * dU2;
@@ -993,17 +917,17 @@ __device__ __forceinline__ void fp64_collide(const LbmParams& P, const CollideCo
       d[2 * k + 1] = d[2 * k + 2] + (BdS + t);
       d[2 * k + 2] = dq + (BdS - t);
     }
-    if (cov) slot_force<T>(P, e, 0, T(1), Ux - Vx, Uy - Vy, Uz - Vz, h + CC_F);
+    if (cov) P.force(e, 0, T(1), Ux - Vx, Uy - Vy, Uz - Vz, h + CC_F);
   } else {
     // the cell's slots; the second one's record is read only when present
     T r0[4] = {T(0), T(0), T(0), T(0)}, r1[4] = {T(0), T(0), T(0), T(0)};
     bool has1 = false;
     T omB = T(1);
     if (cov) {
-      ld4(static_cast<const T*>(P.slot_V) + 4LL * e, r0);
+      ld4(P.V + 4LL * e, r0);
       has1 = neg_flag(r0[3]);
       r0[3] = magnitude(r0[3]);
-      if (has1) ld4(static_cast<const T*>(P.slot_V) + 4LL * (P.slot_cap + e), r1);
+      if (has1) ld4(P.V + 4LL * (P.cap + e), r1);
       T B = r0[3] + r1[3];
       if (B > T(1)) B = T(1);
       omB = T(1) - B;
@@ -1053,7 +977,7 @@ __device__ __forceinline__ void fp64_collide(const LbmParams& P, const CollideCo
       d[2 * k + 1] = SYM + ANT;
       d[2 * k + 2] = SYM - ANT;
     }
-    if (cov) slot_force<T>(P, e, 0, B0, Ux - Vx, Uy - Vy, Uz - Vz, h + CC_F);
+    if (cov) P.force(e, 0, B0, Ux - Vx, Uy - Vy, Uz - Vz, h + CC_F);
     // slot 1 (a cell shared by two particles: rare), on its own
     if (__any_sync(0xffffffffu, has1) && has1) {
       const T Wx = r1[0], Wy = r1[1], Wz = r1[2], B1 = r1[3];
@@ -1074,129 +998,157 @@ __device__ __forceinline__ void fp64_collide(const LbmParams& P, const CollideCo
         d[2 * k + 1] += BdS + BA;
         d[2 * k + 2] += BdS - BA;
       }
-      slot_force<T>(P, e, 1, B1, Ux - Wx, Uy - Wy, Uz - Wz, h + CC_F);
+      P.force(e, 1, B1, Ux - Wx, Uy - Wy, Uz - Wz, h + CC_F);
     }
   }
 }
 
-// The producer warp lists the cells of a tile into the tile's stage: the
-// live cells' positions (r << 16 | x) in three groups, each in cell order:
-// uncovered cells, covered cells, and covered cells of one particle with
-// B = 1 (the full mask), with each covered cell's slot index (-1 for an
-// uncovered cell); hdr[0] = number of uncovered cells, hdr[1] = number of
-// live cells, hdr[2] = index of the first cell of the third group.  Two
-// warp-wide passes over the tile's coverage words (the group sizes, then the
-// entries); the lanes load the words 32 at a time and the rounds take them by
-// shuffles.
-__device__ __forceinline__ void fp64_list_tile(const LbmParams& P, int tile, int nw,
-                                               int* lst_cell, int* lst_slot, int* hdr,
-                                               int lane) {
+// ---- the FP64 form's two kernels.  Cells without particles and covered cells
+// need code of 1,200 to 2,500 instructions each; run together, whether as
+// bodies of their own or as one with branches, they miss in the instruction
+// cache on a quarter of the cycles and more (settle512: 14.1 to 27 ms for the
+// collision).  So the uncovered cells have a kernel (staged rows), and the
+// covered cells, which the slot table lists in cell order, another that
+// gathers their 19 values.  (The first kernel copying them out of its stages
+// for the second, in slot order, took as much longer as the second gained.)
+
+// The uncovered cells of a tile are listed into the tile's stage in cell order
+// (r << 16 | x), hdr[0] = their number.  Lane k holds coverage word k of the
+// tile, loaded a tile ahead; the words' places come from a warp scan, so the
+// rounds that write the entries of a word do not depend on one another.  (A
+// loop that carried the counts from word to word took 4.4 us for a tile of 256
+// cells and bound the kernel.)
+__device__ __forceinline__ int warp_scan(int v, int lane) {  // inclusive
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += t;
+  }
+  return v;
+}
+// A tile: nr whole x-rows from row0, or one segment of a row
+struct Tile {
+  int row0, nr;   // rows
+  int xw, words;  // first word within the row, words in all (at most 32)
+  size_t word0;   // index of the first coverage word
+};
+__device__ __forceinline__ Tile tile_at(const LbmParams& P, int t, int nrows) {
+  Tile T;
   const Grid& g = P.g;
-  const size_t word0 = (size_t)tile * P.tile_rows * g.wpr;
+  if (P.nseg == 1) {
+    T.row0 = t * P.tile_rows;
+    T.nr = min(P.tile_rows, nrows - T.row0);
+    T.xw = 0;
+    T.words = T.nr * g.wpr;
+  } else {
+    T.row0 = (int)P.div_seg.div((unsigned)t);
+    T.nr = 1;
+    T.xw = (t - T.row0 * P.nseg) * P.seg_words;
+    T.words = min(P.seg_words, g.wpr - T.xw);
+  }
+  T.word0 = (size_t)T.row0 * g.wpr + T.xw;
+  return T;
+}
+// m_l: the lane's coverage word
+__device__ __forceinline__ void list_uncovered(const LbmParams& P, const Tile& T, uint32_t m_l,
+                                               int* lst, int* hdr, int lane) {
+  const Grid& g = P.g;
+  uint32_t u_l = 0u;  // uncovered live cells of the lane's word
+  int ent_l = 0;
+  if (lane < T.words) {
+    const int r = T.nr == 1 ? 0 : (int)g.div_wpr.div((unsigned)lane);
+    const int x0 = (T.xw + lane - r * g.wpr) * 32, n = g.nx - x0;
+    u_l = (n >= 32 ? 0xffffffffu : (1u << (n > 0 ? n : 0)) - 1u) & ~m_l;
+    ent_l = (r << 16) | x0;
+  }
+  const int cnt = __popc(u_l), incl = warp_scan(cnt, lane), first_l = incl - cnt;
   const unsigned below = (1u << lane) - 1u;
-  int pu = 0, pc = 0, pf = 0, tot_u = 0, tot_c = 0;
-  // two passes over the words (counts, then entries), 32 words at a time:
-  // lane k loads word w0 + k and the rounds take them by shuffles, so each
-  // round issues its loads together
-  for (int pass = 0; pass < 2; ++pass) {
-    if (pass == 1) {
-      pc = tot_u;  // the covered cells follow all uncovered ones
-      pf = tot_u + tot_c;  // and the full ones follow them
-      pu = 0;
-    }
-    for (int w0 = 0; w0 < nw; w0 += 32) {
-      const int kmax = min(32, nw - w0);
-      const bool own = P.mask && lane < kmax;
-      const uint32_t m_l = own ? __ldg(&P.mask[word0 + w0 + lane]) : 0u;
-      const uint32_t f_l = (own && P.full) ? __ldg(&P.full[word0 + w0 + lane]) : 0u;
-      const int b_l = (own && pass == 1) ? __ldg(&P.base[word0 + w0 + lane]) : 0;
-      for (int k = 0; k < kmax; ++k) {
-        const int w = w0 + k;
-        const int r = (int)g.div_wpr.div((unsigned)w);
-        const int xr = (w - r * g.wpr) * 32 + lane;
-        const bool live = xr < g.nx;
-        const uint32_t m = __shfl_sync(0xffffffffu, m_l, k);
-        const uint32_t fm = __shfl_sync(0xffffffffu, f_l, k) & m;
-        const bool cv = live && ((m >> lane) & 1u);
-        const bool fl = live && ((fm >> lane) & 1u);
-        const unsigned bu = __ballot_sync(0xffffffffu, live && !cv);
-        const unsigned bc = __ballot_sync(0xffffffffu, cv && !fl);
-        const unsigned bf = __ballot_sync(0xffffffffu, fl);
-        if (pass == 0) {
-          pu += __popc(bu);
-          pc += __popc(bc);
-          continue;
-        }
-        const int base = __shfl_sync(0xffffffffu, b_l, k);
-        if (live) {
-          const int pos = fl   ? pf + __popc(bf & below)
-                          : cv ? pc + __popc(bc & below)
-                               : pu + __popc(bu & below);
-          lst_cell[pos] = (r << 16) | xr;
-          int e = -1;
-          if (cv) {
-            e = base + __popc(m & below);
-            if (e >= P.slot_cap) e = -1;  // never the case: the mapping sized the slots
-          }
-          lst_slot[pos] = e;
-        }
-        pu += __popc(bu);
-        pc += __popc(bc);
-        pf += __popc(bf);
-      }
-    }
-    if (pass == 0) {
-      tot_u = pu;
-      tot_c = pc;
-    }
+#pragma unroll 4
+  for (int k = 0; k < T.words; ++k) {
+    const uint32_t u = __shfl_sync(0xffffffffu, u_l, k);
+    const int first = __shfl_sync(0xffffffffu, first_l, k);
+    const int ent = __shfl_sync(0xffffffffu, ent_l, k);
+    if ((u >> lane) & 1u) lst[first + __popc(u & below)] = ent + lane;
   }
-  if (lane == 0) {
-    hdr[0] = tot_u;
-    hdr[1] = pf;  // after the second pass: every live cell
-    hdr[2] = tot_u + tot_c;
-  }
+  if (lane == 31) hdr[0] = incl;
 }
 
-// Staged FP64 kernel with compacted warps: the producer warp and the ring of
-// staged rows are those of lbm_bulk_kernel, and the producer also lists each
-// tile's cells into the tile's stage (fp64_list_tile) before it arrives on
-// the stage's full barrier (count 2: its expect-tx arrival and this one), so
-// the consumers find the list with the data.  Consumer warps take 32 list
-// entries at a time and need no barrier among themselves.
+// Range of the fixed-point form for a warp's cells: E of each lane; lanes
+// outside it (slow) go to the FP64 form, exactly quiescent cells without
+// forces get zeros (quiet)
+struct FxRange {
+  int E;
+  bool slow, quiet;
+};
+__device__ __forceinline__ FxRange fx_range(int top, int E0, int add, int emax) {
+  FxRange r;
+  r.E = fx_exponent(top, E0) + add;
+  r.slow = r.E > emax;
+  r.quiet = E0 <= FX_EMIN && top == 0;
+  if (r.slow) r.E = E0;  // the lane's fixed-point result is not used
+  return r;
+}
+
+// Staged kernel of the cells without particles.  A copy warp streams each
+// tile's rows (or its segment of a row, with two cells more on either side) of
+// the 19 directions into a ring of stages by bulk copies on mbarriers; a list
+// warp lists the tile's cells into the stage and arrives on the same full
+// barrier (count 2: the expect-tx arrival and this one).  One warp for
+// both bound the kernel on narrow rows.  Tiles have at most 256 cells: with
+// rows of 512 the ring holds two of them only.
+//
+// Consumers: a tile has one ticket per coverage word, at least its chunks;
+// warps take tickets in order, each a chunk of 32 list entries of a tile (or
+// none, beyond the tile's chunks), wait for the tile's stage and hand it back
+// ticket by ticket.  A warp claims its next ticket while it works on one.
+// (Every warp visiting every tile cost a wait and a claim per warp and tile,
+// and left warps idle where a tile's chunks are not a multiple of them.)
 template <int MODE, int WALLS>
-__global__ void __launch_bounds__(BULK_THREADS, 1) lbm_fp64_kernel(LbmParams P) {
+__global__ void __launch_bounds__(F64_THREADS, 1) lbm_fp64_kernel(LbmParams P) {
   using T = double;
   extern __shared__ __align__(128) unsigned char bulk_smem[];
   const Grid& g = P.g;
   unsigned long long* full = reinterpret_cast<unsigned long long*>(bulk_smem);
   unsigned long long* empty = full + BULK_MAX_STAGES;
   const int S = P.stages, TR = P.tile_rows, nxp = g.nxp;
-  const int C = TR * nxp;  // elements per direction in a tile
+  const bool seg = P.nseg > 1;
+  const int rowlen = seg ? 32 * P.seg_words + 4 : nxp;  // staged cells per row
+  const int C = TR * rowlen;  // elements per direction in a stage
+  const int words = seg ? P.seg_words : TR * g.wpr;  // of a whole tile
   const size_t stage_elems = (size_t)Q * C;
-  // the barriers, the step's collision coefficients, the ring
-  CollideCoef<double>* coef = reinterpret_cast<CollideCoef<double>*>(bulk_smem + BULK_BAR_BYTES);
-  T* ring = reinterpret_cast<T*>(bulk_smem + BULK_BAR_BYTES + F64_COEF_BYTES);
-  // per stage: header (2 ints, padded to 4), cells, slot indices
+  // the barriers, the ticket, the forcing table, the ring, and per stage a
+  // header (1 int, padded to 4) and the list
+  unsigned* ticket = reinterpret_cast<unsigned*>(bulk_smem + BULK_BAR_BYTES);
+  FxRow* rows = reinterpret_cast<FxRow*>(bulk_smem + BULK_BAR_BYTES + F64_TICKET_BYTES);
+  T* ring = reinterpret_cast<T*>(bulk_smem + BULK_BAR_BYTES + F64_TICKET_BYTES + F64_FX_BYTES);
   int* lists = reinterpret_cast<int*>(ring + S * stage_elems);
-  const size_t list_ints = 4 + 2 * (size_t)C;
+  const size_t list_ints = 4 + 32 * (size_t)words;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nrows = g.ny * g.nz;
   {
-    constexpr int NV = (int)(sizeof(CollideCoef<double>) / sizeof(double2));
-    const double2* src = reinterpret_cast<const double2*>(&P.sc->d);
-    for (int i = threadIdx.x; i < NV; i += blockDim.x) reinterpret_cast<double2*>(coef)[i] = src[i];
+    constexpr int NR = (int)(sizeof(FxRow) * FX_ROWS / sizeof(double2));
+    const double2* srow = reinterpret_cast<const double2*>(P.sc->fx);
+    for (int i = threadIdx.x; i < NR; i += blockDim.x) reinterpret_cast<double2*>(rows)[i] = srow[i];
   }
   if (threadIdx.x == 0) {
+    *ticket = 0u;
     for (int s = 0; s < S; ++s) {
       mbar_init(&full[s], 2);
-      mbar_init(&empty[s], BULK_CONSUMER_WARPS);
+      mbar_init(&empty[s], (unsigned)words);
     }
     mbar_fence_init();
   }
   __syncthreads();
 
-  if (warp == BULK_CONSUMER_WARPS) {
-    // ---- producer
+  if (warp >= F64_CONSUMER_WARPS) {
+    const bool copy = warp == F64_CONSUMER_WARPS;
+    // a tile's coverage words, loaded a tile ahead
+    auto words_of = [&](int t) {
+      if (copy || !P.mask || t >= P.ntiles) return 0u;
+      const Tile tl = tile_at(P, t, nrows);
+      return lane < tl.words ? __ldg(&P.mask[tl.word0 + lane]) : 0u;
+    };
+    uint32_t next = words_of(blockIdx.x);
     int issued = 0;
     for (int tile = blockIdx.x; tile < P.ntiles; tile += gridDim.x) {
       const int s = issued % S;
@@ -1205,39 +1157,68 @@ __global__ void __launch_bounds__(BULK_THREADS, 1) lbm_fp64_kernel(LbmParams P) 
         if (lane == 0) atomicOr(P.status, ST_TIMEOUT);
         break;
       }
-      const int row0 = tile * TR;
-      const int nr = min(TR, nrows - row0);
-      if (lane == 0) mbar_expect_tx(&full[s], (unsigned)(Q * nr * nxp * sizeof(T)));
-      __syncwarp();
-      T* st = ring + s * stage_elems;
-      for (int j = lane; j < Q * nr; j += 32) {
-        const int q = j / nr, r = j - q * nr;
-        const int row = row0 + r;
-        const int z = (int)g.div_ny.div((unsigned)row);
-        const int y = row - z * g.ny;
-        int sy = y, sz = z, sq = q;
-        if (MODE != 1 && q > 0) {
-          const int k = (q - 1) >> 1, sg = qsign(q);
-          sy -= sg * cky(k);
-          sz -= sg * ckz(k);
-          sy = sy < 0 ? sy + g.ny : (sy >= g.ny ? sy - g.ny : sy);
-          sz = sz < 0 ? sz + g.nz : (sz >= g.nz ? sz - g.nz : sz);
-          if (MODE == 2) sq = q + sg;  // AA odd: the opposite direction's array
+      const Tile tl = tile_at(P, tile, nrows);
+      if (copy) {
+        // ---- the copies: lane q < 19 takes direction q.  Staged cell x of
+        // row r at (q TR + r) rowlen + x - xs
+        const int xs = seg ? 32 * tl.xw - 2 : 0;
+        const int xa = xs > 0 ? xs : 0;
+        const int xb = seg ? min(32 * (tl.xw + tl.words) + 2, nxp) : nxp;
+        const unsigned row_bytes = (unsigned)((xb - xa) * sizeof(T));
+        if (lane == 0) mbar_expect_tx(&full[s], (unsigned)(Q * tl.nr) * row_bytes);
+        __syncwarp();
+        if (lane < Q) {
+          const int q = lane;
+          int cy = 0, cz = 0, sq = q;
+          if (MODE != 1 && q > 0) {
+            const int k = (q - 1) >> 1, sg = qsign(q);
+            cy = sg * cky(k);
+            cz = sg * ckz(k);
+            if (MODE == 2) sq = q + sg;  // AA odd: the opposite direction's array
+          }
+          const T* base = static_cast<const T*>(P.src) + (size_t)sq * g.ncell + xa;
+          T* dst = ring + s * stage_elems + (size_t)q * C + (xa - xs);
+          int z = (int)g.div_ny.div((unsigned)tl.row0);
+          int y = tl.row0 - z * g.ny;
+          // rows that follow one another in memory go in one copy
+          int r0 = 0, first = 0, prev = -2;
+          for (int r = 0; r <= tl.nr; ++r) {
+            int src = -1;
+            if (r < tl.nr) {
+              int sy = y - cy, sz = z - cz;
+              sy = sy < 0 ? sy + g.ny : (sy >= g.ny ? sy - g.ny : sy);
+              sz = sz < 0 ? sz + g.nz : (sz >= g.nz ? sz - g.nz : sz);
+              src = sz * g.ny + sy;
+              if (++y == g.ny) {
+                y = 0;
+                ++z;
+              }
+            }
+            if (src != prev + 1 || r == tl.nr) {
+              if (r > r0)
+                bulk_copy_g2s(dst + (size_t)r0 * rowlen, base + (size_t)first * nxp,
+                              (unsigned)(r - r0) * row_bytes, &full[s]);
+              r0 = r;
+              first = src;
+            }
+            prev = src;
+          }
         }
-        const T* src = static_cast<const T*>(P.src) + (size_t)sq * g.ncell +
-                       ((size_t)sz * g.ny + sy) * nxp;
-        bulk_copy_g2s(st + ((size_t)q * TR + r) * nxp, src, (unsigned)(nxp * sizeof(T)),
-                      &full[s]);
+        __syncwarp();
+      } else {
+        // ---- the list
+        int* ls = lists + s * list_ints;
+        const uint32_t cur = next;
+        next = words_of(tile + (int)gridDim.x);
+        list_uncovered(P, tl, cur, ls + 4, ls, lane);
+        __threadfence_block();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&full[s]);  // release: the list is visible with the data
       }
-      int* ls = lists + s * list_ints;
-      fp64_list_tile(P, tile, nr * g.wpr, ls + 4, ls + 4 + C, ls, lane);
-      __threadfence_block();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&full[s]);  // release: the list is visible with the data
       ++issued;
     }
     // no copy may land after the block has exited
-    for (int j = issued - S < 0 ? 0 : issued - S; j < issued; ++j)
+    for (int j = issued - S < 0 ? 0 : issued - S; copy && j < issued; ++j)
       if (!mbar_wait(&full[j % S], (unsigned)(j / S) & 1u)) {
         if (lane == 0) atomicOr(P.status, ST_TIMEOUT);
       }
@@ -1246,65 +1227,268 @@ __global__ void __launch_bounds__(BULK_THREADS, 1) lbm_fp64_kernel(LbmParams P) 
 
   // ---- consumers
 #define SRC(q) static_cast<const T*>(P.srcq[q])
-  int it = 0;
-  for (int tile = blockIdx.x; tile < P.ntiles; tile += gridDim.x, ++it) {
+  const int E0 = P.sc->fx_E0;
+  auto claim = [&]() {
+    unsigned t = 0;
+    if (lane == 0) t = atomicAdd(ticket, 1u);
+    return t;  // in lane 0
+  };
+  unsigned mine = claim();
+  for (;;) {
+    const unsigned tk = __shfl_sync(0xffffffffu, mine, 0);
+    mine = claim();
+    const int it = (int)P.div_words.div(tk);
+    const int ch = (int)tk - it * words;
+    const int tile = (int)blockIdx.x + it * (int)gridDim.x;
+    if (tile >= P.ntiles) break;
     const int s = it % S;
     if (!mbar_wait(&full[s], (unsigned)(it / S) & 1u)) {
       if (lane == 0) atomicOr(P.status, ST_TIMEOUT);
       break;
     }
-    const T* st = ring + s * stage_elems;
     const int* ls = lists + s * list_ints;
-    const int tot_u = ls[0], L = ls[1], full0 = ls[2];
-    const int* lst_cell = ls + 4;
-    const int* lst_slot = ls + 4 + C;
-    const int row0 = tile * TR;
-    const int nch = (L + 31) / 32;
-    // the covered chunks come last in every tile: the chunk a warp starts
-    // with turns by 3 from tile to tile (3 and 8 are coprime), so every
-    // warp takes its share of them and none runs ahead of the ring
-    const int ch0 = (warp + 3 * it) % BULK_CONSUMER_WARPS;
-    for (int ch = ch0; ch < nch; ch += BULK_CONSUMER_WARPS) {
+    const int L = ls[0];
+    if (ch * 32 < L) {
+      const Tile tl = tile_at(P, tile, nrows);
       const int i = ch * 32 + lane;
-      const bool active = i < L;
-      const int ent = lst_cell[active ? i : L - 1];
-      const int e = active ? lst_slot[i] : -1;
-      const int r = ent >> 16, x = ent & 0xffff;
-      const int row = row0 + r;
+      bool act = i < L;
+      const int le = ls[4 + (act ? i : L - 1)];
+      const int r = le >> 16, x = le & 0xffff;
+      const int row = tl.row0 + r;
       const int z = (int)g.div_ny.div((unsigned)row);
       const int y = row - z * g.ny;
       NbrT<WALLS> nb;
-      nb.init(x, y, z, g.nx, g.ny, g.nz, g.nxp, g.wall);
+      nb.init(x, y, z, g.nx, g.ny, g.nz, nxp, g.wall);
       const int cell = nb.idx(0, 0, 0);
-      const int xm = x == 0 ? g.nx - 1 : x - 1, xq = x == g.nx - 1 ? 0 : x + 1;
-      const T* sr = st + (size_t)r * nxp;  // direction q of this row at sr[q * C]
+      // staged index of x - 1, x, x + 1.  A neighbour across the periodic x
+      // face is not in a segment's stage, and a link across a wall takes the
+      // own cell: those lanes, few, replace the staged values from global
+      // memory
+      const int xs = seg ? 32 * tl.xw - 2 : 0;
+      const int i0 = x - xs;
+      int im = (x == 0 ? g.nx : x) - 1 - xs, ip = (x == g.nx - 1 ? 0 : x + 1) - xs;
+      const bool inm = (unsigned)im < (unsigned)rowlen, inp = (unsigned)ip < (unsigned)rowlen;
+      if (!inm) im = i0;
+      if (!inp) ip = i0;
+      const T* sr = ring + s * stage_elems + (size_t)r * rowlen;  // direction q at sr[q * C]
       T d[Q];
-      d[0] = sr[x];
+      d[0] = sr[i0];
+#pragma unroll
+      for (int k = 0; k < 9; ++k) {
+        // qa comes from x - c_x, qb from x + c_x (AA odd: from the opposite
+        // direction's array, staged as such)
+        const int cx = MODE == 1 ? 0 : ckx(k);
+        const int qa = 2 * k + 1, qb = 2 * k + 2;
+        d[qa] = sr[qa * C + (cx > 0 ? im : (cx < 0 ? ip : i0))];
+        d[qb] = sr[qb * C + (cx > 0 ? ip : (cx < 0 ? im : i0))];
+      }
+      const bool at_wall = ((WALLS & 1) && !(nb.ok(-1, 0, 0) && nb.ok(1, 0, 0))) ||
+                           ((WALLS & 2) && !(nb.ok(0, -1, 0) && nb.ok(0, 1, 0))) ||
+                           ((WALLS & 4) && !(nb.ok(0, 0, -1) && nb.ok(0, 0, 1)));
+      if (MODE != 1 && (!inm || !inp || at_wall)) {
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+          const int cx = ckx(k), cy = cky(k), cz = ckz(k);
+          const int qa = 2 * k + 1, qb = 2 * k + 2;
+          const int ga = MODE == 0 ? qa : qb, gb = MODE == 0 ? qb : qa;  // arrays of the links
+          const bool na = cx > 0 ? inm : (cx < 0 ? inp : true);
+          const bool nx = cx > 0 ? inp : (cx < 0 ? inm : true);
+          if (!nb.ok(-cx, -cy, -cz)) d[qa] = ld(SRC(gb) + cell);
+          else if (!na) d[qa] = ld(SRC(ga) + nb.idx(-cx, -cy, -cz));
+          if (!nb.ok(cx, cy, cz)) d[qb] = ld(SRC(ga) + cell);
+          else if (!nx) d[qb] = ld(SRC(gb) + nb.idx(cx, cy, cz));
+        }
+        if constexpr (MODE == 0) apply_open_faces<T, WALLS>(P, nb, z, cell, d);
+      }
+      auto put = [&](int q, T v) {
+        if (act) store_pdf<T, MODE, WALLS>(P, nb, cell, q, v);
+      };
+      const FxRange R = fx_range(fx_top(d), E0, 0, FX_EMAX);
+      if (R.quiet) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) put(q, 0.0);
+        act = false;
+      }
+      const bool live = act, any_slow = __any_sync(0xffffffffu, R.slow);
+      double t[Q];  // a copy: an array whose address is passed lives in memory
+      if (any_slow) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) t[q] = d[q];
+        act = act && !R.slow;
+      }
+      if (__any_sync(0xffffffffu, act) && E0 <= FX_EMAX)
+        fx_collide<FX_FLUID>(P.fx, rows[min(R.E - E0, FX_ROWS - 1)], R.E, d, nullptr,
+                             [](const double*) {}, put);
+      if (any_slow) {
+        fp64_collide<CK_UNCOVERED>(F64Slots{nullptr, nullptr, 0}, &P.sc->d, t, false, -1);
+        act = live && R.slow;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) put(q, t[q]);
+      }
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&empty[s]);
+  }
+}
+
+// Kernel of the covered cells: blocks claim groups of COV_GROUP slot entries
+// (consecutive covered cells), sort them by kind (one particle with B < 1, one
+// with B = 1, two particles) and take each kind's entries 32 at a time, so that
+// the block's warps run the same code at about the same time.  The cells of
+// two particles, few, run the FP64 form.  (Queues per warp, with the next 32
+// cells' values fetched by cp.async, let the kinds interleave in the
+// instruction cache and left each warp partly filled last chunks: 16% slower.)
+constexpr int COV_THREADS = 256, COV_GROUP = 1024;
+constexpr int COV_WARPS = COV_THREADS / 32, COV_ROUNDS = COV_GROUP / COV_THREADS;
+template <int MODE, int WALLS>
+__global__ void __launch_bounds__(COV_THREADS, 2) lbm_fp64_covered_kernel(LbmParams P) {
+  using T = double;
+  const Grid& g = P.g;
+  __shared__ FxRow rows[FX_ROWS];
+  __shared__ int2 lst[COV_GROUP];         // entry, padded cell
+  __shared__ int cnt[3][COV_GROUP / 32];  // per kind and 32 entries: count, then first place
+  __shared__ int tot[3];
+  __shared__ unsigned group, chunk;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned all = 0xffffffffu, below = (1u << lane) - 1u;
+  const int n = (int)min((long long)*P.ncov, P.slot_cap);
+  const F64Slots S{static_cast<const double*>(P.slot_V), static_cast<double*>(P.slot_Fc),
+                   P.slot_cap};
+  const int E0 = P.sc->fx_E0;
+  for (int i = threadIdx.x; i < (int)(sizeof(rows) / sizeof(double2)); i += COV_THREADS)
+    reinterpret_cast<double2*>(rows)[i] = reinterpret_cast<const double2*>(P.sc->fx)[i];
+  for (;;) {
+    __syncthreads();  // the previous group is done
+    if (threadIdx.x == 0) {
+      group = atomicAdd(P.work, 1u);
+      chunk = 0u;
+    }
+    __syncthreads();
+    const long long base = (long long)group * COV_GROUP;
+    if (base >= n) {
+      // each block ends on one claim too many: the last of them resets the
+      // counter for the next launch
+      const unsigned groups = (unsigned)((n + COV_GROUP - 1) / COV_GROUP);
+      if (threadIdx.x == 0 && group == groups + gridDim.x - 1) *P.work = 0u;
+      break;
+    }
+    // ---- kinds (2: B = 1, 1: two particles, 0: other) of the thread's entries
+    int kind[COV_ROUNDS], own[COV_ROUNDS];
+#pragma unroll
+    for (int j = 0; j < COV_ROUNDS; ++j) {
+      const long long e = base + j * COV_THREADS + threadIdx.x;
+      const double B = e < n ? S.V[4 * e + 3] : 0.0;
+      own[j] = e < n ? P.slot_cell[e] : 0;
+      kind[j] = e >= n ? -1 : (neg_flag(B) ? 1 : (B == 1.0 ? 2 : 0));
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const unsigned b = __ballot_sync(all, kind[j] == k);
+        if (lane == 0) cnt[k][j * COV_WARPS + warp] = __popc(b);
+      }
+    }
+    __syncthreads();
+    if (warp < 3) {
+      static_assert(COV_GROUP / 32 == 32, "one lane per count");
+      const int v = cnt[warp][lane], incl = warp_scan(v, lane);
+      cnt[warp][lane] = incl - v;
+      if (lane == 31) tot[warp] = incl;
+    }
+    __syncthreads();
+    const int n0 = tot[0], n1 = tot[1], n2 = tot[2];
+#pragma unroll
+    for (int j = 0; j < COV_ROUNDS; ++j)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const unsigned b = __ballot_sync(all, kind[j] == k);
+        if (kind[j] == k)
+          lst[(k == 0 ? 0 : (k == 1 ? n0 : n0 + n1)) + cnt[k][j * COV_WARPS + warp] +
+              __popc(b & below)] = make_int2(j * COV_THREADS + threadIdx.x, own[j]);
+      }
+    __syncthreads();
+    const int c0 = (n0 + 31) / 32, c1 = (n1 + 31) / 32, c2 = (n2 + 31) / 32;
+    for (;;) {
+      int c = 0;
+      if (lane == 0) c = (int)atomicAdd(&chunk, 1u);
+      c = __shfl_sync(all, c, 0);
+      if (c >= c0 + c1 + c2) break;
+      // the longest first: two particles, mixed, full
+      const int kd = c < c1 ? 1 : (c < c1 + c0 ? 0 : 2);
+      const int first = kd == 0 ? 0 : (kd == 1 ? n0 : n0 + n1);
+      const int num = kd == 0 ? n0 : (kd == 1 ? n1 : n2);
+      const int i = 32 * (kd == 1 ? c : (kd == 0 ? c - c1 : c - c1 - c0)) + lane;
+      bool act = i < num;
+      const int2 le = lst[first + (act ? i : num - 1)];
+      const int e = (int)base + le.x, cell = le.y;
+      double V[4];
+      ld4(S.V + 4LL * e, V);
+      const unsigned row = g.div_wpr.div((unsigned)cell >> 5);
+      const int z = (int)g.div_ny.div(row);
+      NbrT<WALLS> nb;
+      nb.init(cell - (int)row * g.nxp, (int)row - z * g.ny, z, g.nx, g.ny, g.nz, g.nxp, g.wall);
+      T d[Q];
+      d[0] = ld(SRC(0) + cell);
 #pragma unroll
       for (int k = 0; k < 9; ++k) {
         const int cx = ckx(k), cy = cky(k), cz = ckz(k);
         const int qa = 2 * k + 1, qb = 2 * k + 2;
-        const int xa = cx > 0 ? xm : (cx < 0 ? xq : x);  // x - c_x
-        const int xb = cx > 0 ? xq : (cx < 0 ? xm : x);  // x + c_x
         if (MODE == 0) {
-          d[qa] = nb.ok(-cx, -cy, -cz) ? sr[qa * C + xa] : ld(SRC(qb) + cell);
-          d[qb] = nb.ok(cx, cy, cz) ? sr[qb * C + xb] : ld(SRC(qa) + cell);
+          d[qa] = nb.ok(-cx, -cy, -cz) ? ld(SRC(qa) + nb.idx(-cx, -cy, -cz)) : ld(SRC(qb) + cell);
+          d[qb] = nb.ok(cx, cy, cz) ? ld(SRC(qb) + nb.idx(cx, cy, cz)) : ld(SRC(qa) + cell);
         } else if (MODE == 1) {
-          d[qa] = sr[qa * C + x];
-          d[qb] = sr[qb * C + x];
+          d[qa] = ld(SRC(qa) + cell);
+          d[qb] = ld(SRC(qb) + cell);
         } else {
-          d[qa] = nb.ok(-cx, -cy, -cz) ? sr[qa * C + xa] : ld(SRC(qa) + cell);
-          d[qb] = nb.ok(cx, cy, cz) ? sr[qb * C + xb] : ld(SRC(qb) + cell);
+          d[qa] = nb.ok(-cx, -cy, -cz) ? ld(SRC(qb) + nb.idx(-cx, -cy, -cz)) : ld(SRC(qa) + cell);
+          d[qb] = nb.ok(cx, cy, cz) ? ld(SRC(qa) + nb.idx(cx, cy, cz)) : ld(SRC(qb) + cell);
         }
       }
       if constexpr (MODE == 0) apply_open_faces<T, WALLS>(P, nb, z, cell, d);
-      if (ch * 32 + 32 <= tot_u) fp64_collide<CK_UNCOVERED>(P, coef, d, false, -1);
-      else if (ch * 32 >= full0) fp64_collide<CK_FULL>(P, coef, d, e >= 0, e);
-      else fp64_collide<CK_MIXED>(P, coef, d, e >= 0, e);
-      if (active) store_pdfs<T, MODE, WALLS>(P, nb, cell, d);
+      auto put = [&](int q, T v) {
+        if (act) store_pdf<T, MODE, WALLS>(P, nb, cell, q, v);
+      };
+      auto force = [&](const double* F) {
+        if (act) {
+          double* o = S.Fc + 3LL * e;
+          o[0] = F[0];
+          o[1] = F[1];
+          o[2] = F[2];
+        }
+      };
+      int top = fx_top(d);
+      top = fx_top_velocity(top, V, kd == 2 ? FX_VBITS_FULL : FX_VBITS_MIXED);
+      FxRange R = fx_range(top, E0, kd == 2 ? 0 : 1, FX_EMAX_SOLID);
+      if (kd == 1) {
+        R.slow = true;
+        R.quiet = false;
+      }
+      if (R.quiet) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) put(q, 0.0);
+        const double zero[3] = {0.0, 0.0, 0.0};
+        force(zero);
+        act = false;
+      }
+      const bool live = act, any_slow = __any_sync(all, R.slow);
+      double t[Q];  // a copy: an array whose address is passed lives in memory
+      if (any_slow) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) t[q] = d[q];
+        act = act && !R.slow;
+      }
+      if (__any_sync(all, act) && E0 <= FX_EMAX_SOLID) {
+        const FxRow& row = rows[min(R.E - E0, FX_ROWS - 1)];
+        if (kd == 2) fx_collide<FX_FULL>(P.fx, row, R.E, d, V, force, put);
+        else fx_collide<FX_MIXED>(P.fx, row, R.E, d, V, force, put);
+      }
+      if (any_slow) {
+        const bool cov = live && R.slow;
+        if (kd == 2) fp64_collide<CK_FULL>(S, &P.sc->d, t, cov, cov ? e : -1);
+        else fp64_collide<CK_MIXED>(S, &P.sc->d, t, cov, cov ? e : -1);
+        act = cov;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) put(q, t[q]);
+      }
     }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(&empty[s]);
   }
 #undef SRC
 }
@@ -1467,28 +1651,15 @@ __global__ void sums_final_kernel(int nparts, const double* __restrict__ partial
 
 }  // namespace
 
-template <typename T>
-size_t lbm_dyn_smem() {
-  return kFP64<T> ? lbm_smem_bytes<T>() : 0;
-}
-
-template <typename T, int W>
+template <int W>
 int configure_walls(int optin) {
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  const int sm = (int)lbm_dyn_smem<T>();
   int bad = 0;
-  bad |= cudaFuncSetAttribute(lbm_kernel<T, 0, W>, a, sm) != cudaSuccess;
-  bad |= cudaFuncSetAttribute(lbm_kernel<T, 1, W>, a, sm) != cudaSuccess;
-  bad |= cudaFuncSetAttribute(lbm_kernel<T, 2, W>, a, sm) != cudaSuccess;
-  if constexpr (!kFP64<T>) {  // FP64 stages through lbm_fp64_kernel
-    bad |= cudaFuncSetAttribute(lbm_bulk_kernel<T, 0, W>, a, optin) != cudaSuccess;
-    bad |= cudaFuncSetAttribute(lbm_bulk_kernel<T, 1, W>, a, optin) != cudaSuccess;
-    bad |= cudaFuncSetAttribute(lbm_bulk_kernel<T, 2, W>, a, optin) != cudaSuccess;
-  } else {
-    bad |= cudaFuncSetAttribute(lbm_fp64_kernel<0, W>, a, optin) != cudaSuccess;
-    bad |= cudaFuncSetAttribute(lbm_fp64_kernel<1, W>, a, optin) != cudaSuccess;
-    bad |= cudaFuncSetAttribute(lbm_fp64_kernel<2, W>, a, optin) != cudaSuccess;
-  }
+  bad |= cudaFuncSetAttribute(lbm_bulk_kernel<float, 1, W>, a, optin) != cudaSuccess;
+  bad |= cudaFuncSetAttribute(lbm_bulk_kernel<float, 2, W>, a, optin) != cudaSuccess;
+  bad |= cudaFuncSetAttribute(lbm_fp64_kernel<0, W>, a, optin) != cudaSuccess;
+  bad |= cudaFuncSetAttribute(lbm_fp64_kernel<1, W>, a, optin) != cudaSuccess;
+  bad |= cudaFuncSetAttribute(lbm_fp64_kernel<2, W>, a, optin) != cudaSuccess;
   return bad;
 }
 
@@ -1503,24 +1674,13 @@ static int smem_optin() {
 int lbm_configure() {
   const int o = smem_optin();
   if (o <= 0) return 1;
-  return configure_walls<float, 0>(o) | configure_walls<float, 1>(o) |
-         configure_walls<float, 7>(o) | configure_walls<double, 0>(o) |
-         configure_walls<double, 1>(o) | configure_walls<double, 7>(o) |
-         configure_walls<df, 0>(o) | configure_walls<df, 1>(o) | configure_walls<df, 7>(o);
+  return configure_walls<0>(o) | configure_walls<1>(o) | configure_walls<7>(o);
 }
 
-// tiles of whole x-rows: 256 cells (tile_rows rows) when the padded row
-// divides 256, else one row; as many stages as fit the per-block budget
-// (FP32: two blocks per SM; FP64: one block next to the solid-operator
-// scratch).  The staged kernel serves FP64 (FP64-pipe bound: it frees the
-// warps from load latency) and the FP32 AA pattern; FP32 pull streaming runs
-// faster on the one-cell-per-thread kernel, whose 32 resident warps per SM
-// keep enough loads in flight.  Returns 0 and leaves plan.stages = 0 when
-// the one-cell-per-thread kernel is to be used.
 template <typename T, int W>
 const void* bulk_fn() {
-  if constexpr (kFP64<T>) return (const void*)lbm_fp64_kernel<0, W>;
-  else return (const void*)lbm_bulk_kernel<T, 0, W>;
+  if constexpr (sizeof(T) == 8) return (const void*)lbm_fp64_kernel<0, W>;
+  else return (const void*)lbm_bulk_kernel<T, 1, W>;
 }
 template <typename T>
 const void* bulk_fn_w(int w) {
@@ -1544,8 +1704,8 @@ template <typename T>
 int cell_prefetch_ahead(const Grid& g, int* ahead) {
   const int w = g.wall[0] | (g.wall[1] << 1) | (g.wall[2] << 2);
   int per_sm = 0, dev = 0, nsm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cell_fn_w<T>(w), LBM_THREADS,
-                                                    lbm_dyn_smem<T>()) != cudaSuccess ||
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cell_fn_w<T>(w), LBM_THREADS, 0) !=
+          cudaSuccess ||
       cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return 1;
@@ -1553,6 +1713,13 @@ int cell_prefetch_ahead(const Grid& g, int* ahead) {
   return 0;
 }
 
+// Tiles of the staged kernels: 256 cells (tile_rows rows) when the padded row
+// divides 256, else one row, in FP64 cut into segments of at most 8 words; as
+// many stages as fit the per-block budget (FP32: two blocks per SM; FP64: one
+// block, next to its forcing table and cell lists).  They serve FP64 and the
+// FP32 AA pattern; FP32 pull streaming runs faster on the one-cell-per-thread
+// kernel, whose 32 resident warps per SM keep enough loads in flight.  Leaves
+// plan.stages = 0 where that kernel is to be used.
 int lbm_plan(const Grid& g, int prec, int aa, LbmPlan* plan) {
   *plan = LbmPlan{};
   const int fp32 = prec == PREC_FP32;
@@ -1567,74 +1734,109 @@ int lbm_plan(const Grid& g, int prec, int aa, LbmPlan* plan) {
   if (optin <= 0) return 1;
   const size_t esz = fp32 ? sizeof(float) : sizeof(double);
   const int TR = (g.nxp <= 256 && 256 % g.nxp == 0) ? 256 / g.nxp : 1;
-  const size_t stage = (size_t)Q * TR * g.nxp * esz;
-  // FP64 (compacted warps): per stage the tile's cell list and slot indices
-  // with a 16-byte header
-  const size_t list_stage = prec == PREC_FP64 ? (size_t)8 * TR * g.nxp + 16 : 0;
-  const size_t extra = BULK_BAR_BYTES + (prec == PREC_FP64 ? F64_COEF_BYTES : 0);
-  const size_t budget = prec == PREC_FP64 ? (size_t)optin : (size_t)100 * 1024;
-  if (budget <= extra) return 0;
+  // FP64: rows of more than 8 words in equal segments (each staged with two
+  // cells more on either side); per stage the tile's cell list with a 16-byte
+  // header
+  const bool f64 = prec == PREC_FP64;
+  const int nseg = f64 ? (g.wpr + 7) / 8 : 1;
+  const int seg_words = (g.wpr + nseg - 1) / nseg;
+  const int row_cells = nseg > 1 ? 32 * seg_words + 4 : g.nxp;
+  const int tile_cells = nseg > 1 ? 32 * seg_words : TR * g.nxp;
+  const size_t stage = (size_t)Q * TR * row_cells * esz;
+  const size_t list_stage = f64 ? (size_t)4 * tile_cells + 16 : 0;
+  const size_t extra = BULK_BAR_BYTES + (f64 ? F64_TICKET_BYTES + F64_FX_BYTES : 0);
+  const size_t budget = f64 ? (size_t)optin : (size_t)100 * 1024;
+  if (budget <= extra) return f64;
   size_t S = (budget - extra) / (stage + list_stage);
   if (S > BULK_MAX_STAGES) S = BULK_MAX_STAGES;
   if (S < 2) {
-    if (extra + 2 * (stage + list_stage) > (size_t)optin) return 0;
+    if (extra + 2 * (stage + list_stage) > (size_t)optin) return f64;
     S = 2;
   }
   const size_t smem = extra + S * (stage + list_stage);
   const int w = g.wall[0] | (g.wall[1] << 1) | (g.wall[2] << 2);
-  const void* fn = prec == PREC_FP32 ? bulk_fn_w<float>(w)
-                   : prec == PREC_DF ? bulk_fn_w<df>(w)
-                                     : bulk_fn_w<double>(w);
+  const void* fn = f64 ? bulk_fn_w<double>(w) : bulk_fn_w<float>(w);
   int per_sm = 0, dev = 0, nsm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, BULK_THREADS, smem) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+          &per_sm, fn, f64 ? F64_THREADS : BULK_THREADS, smem) !=
           cudaSuccess ||
       cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return 1;
-  if (per_sm < 1) return 0;
+  if (per_sm < 1) return f64;  // FP64 has no other kernel
   const long long nrows = (long long)g.ny * g.nz;
   plan->tile_rows = TR;
-  plan->ntiles = (int)((nrows + TR - 1) / TR);
+  plan->ntiles = (int)(nseg > 1 ? nrows * nseg : (nrows + TR - 1) / TR);
+  plan->nseg = nseg;
+  plan->cov_blocks = 2 * nsm;
+  plan->seg_words = seg_words;
+  plan->div_seg = make_fastdiv((unsigned)nseg);
   plan->stages = (int)S;
   plan->smem = smem;
+  plan->div_words = make_fastdiv((unsigned)(tile_cells / 32));
   const long long blocks = (long long)nsm * per_sm;
   plan->blocks = (int)(blocks < plan->ntiles ? blocks : plan->ntiles);
   return 0;
 }
 
-template <typename T, int W>
-void launch_lbm_t(const LbmParams& P, int mode, unsigned grid, cudaStream_t s) {
-  if (P.stages > 0 && kFP64<T>) {
-    const size_t sm = P.smem;
-    if (mode == 0) lbm_fp64_kernel<0, W><<<P.blocks, BULK_THREADS, sm, s>>>(P);
-    else if (mode == 1) lbm_fp64_kernel<1, W><<<P.blocks, BULK_THREADS, sm, s>>>(P);
-    else lbm_fp64_kernel<2, W><<<P.blocks, BULK_THREADS, sm, s>>>(P);
+// The two kernels work on different cells (every value is read and written by
+// one cell only, in place or not), so they may run side by side.  They do where
+// the staged kernel has no more tiles than SMs and neither fills the device
+// (32^3: 20.1 us instead of 27.3); on larger grids the second kernel's blocks
+// keep the staged kernel's, one per SM, from starting (settle512: 15.5 ms
+// instead of 13.7).
+template <int MODE, int W>
+void launch_fp64(const LbmParams& P, size_t sm, const LbmFork& fk, cudaStream_t s) {
+  if (!P.mask) {
+    lbm_fp64_kernel<MODE, W><<<P.blocks, F64_THREADS, sm, s>>>(P);
     return;
   }
-  if constexpr (!kFP64<T>) {
-    if (P.stages > 0) {
-      const size_t sm = P.smem;
-      if (mode == 0) lbm_bulk_kernel<T, 0, W><<<P.blocks, BULK_THREADS, sm, s>>>(P);
-      else if (mode == 1) lbm_bulk_kernel<T, 1, W><<<P.blocks, BULK_THREADS, sm, s>>>(P);
-      else lbm_bulk_kernel<T, 2, W><<<P.blocks, BULK_THREADS, sm, s>>>(P);
-      return;
-    }
+  const bool beside = fk.side && P.ntiles <= P.blocks;
+  const cudaStream_t side = beside ? fk.side : s;
+  if (beside) {
+    cudaEventRecord(fk.fork, s);
+    cudaStreamWaitEvent(side, fk.fork, 0);
   }
-  const size_t sm = lbm_dyn_smem<T>();
-  if (mode == 0) lbm_kernel<T, 0, W><<<grid, LBM_THREADS, sm, s>>>(P);
-  else if (mode == 1) lbm_kernel<T, 1, W><<<grid, LBM_THREADS, sm, s>>>(P);
-  else lbm_kernel<T, 2, W><<<grid, LBM_THREADS, sm, s>>>(P);
+  lbm_fp64_kernel<MODE, W><<<P.blocks, F64_THREADS, sm, s>>>(P);
+  lbm_fp64_covered_kernel<MODE, W><<<P.cov_blocks, COV_THREADS, 0, side>>>(P);
+  if (beside) {
+    cudaEventRecord(fk.join, side);
+    cudaStreamWaitEvent(s, fk.join, 0);
+  }
+}
+
+template <typename T, int W>
+void launch_lbm_t(const LbmParams& P, int mode, unsigned grid, const LbmFork& fk,
+                  cudaStream_t s) {
+  const size_t sm = P.smem;
+  if constexpr (sizeof(T) == 8 && !kDF<T>) {
+    if (mode == 0) launch_fp64<0, W>(P, sm, fk, s);
+    else if (mode == 1) launch_fp64<1, W>(P, sm, fk, s);
+    else launch_fp64<2, W>(P, sm, fk, s);
+  } else {
+    if constexpr (!kDF<T>) {  // plan.stages > 0: the AA pattern
+      if (P.stages > 0) {
+        if (mode == 1) lbm_bulk_kernel<T, 1, W><<<P.blocks, BULK_THREADS, sm, s>>>(P);
+        else lbm_bulk_kernel<T, 2, W><<<P.blocks, BULK_THREADS, sm, s>>>(P);
+        return;
+      }
+    }
+    if (mode == 0) lbm_kernel<T, 0, W><<<grid, LBM_THREADS, 0, s>>>(P);
+    else if (mode == 1) lbm_kernel<T, 1, W><<<grid, LBM_THREADS, 0, s>>>(P);
+    else lbm_kernel<T, 2, W><<<grid, LBM_THREADS, 0, s>>>(P);
+  }
 }
 
 template <typename T>
-void launch_lbm_w(const LbmParams& P, int mode, unsigned grid, cudaStream_t s) {
+void launch_lbm_w(const LbmParams& P, int mode, unsigned grid, const LbmFork& fk,
+                  cudaStream_t s) {
   const int w = P.g.wall[0] | (P.g.wall[1] << 1) | (P.g.wall[2] << 2);
-  if (w == 0) launch_lbm_t<T, 0>(P, mode, grid, s);
-  else if (w == 1) launch_lbm_t<T, 1>(P, mode, grid, s);
-  else launch_lbm_t<T, 7>(P, mode, grid, s);
+  if (w == 0) launch_lbm_t<T, 0>(P, mode, grid, fk, s);
+  else if (w == 1) launch_lbm_t<T, 1>(P, mode, grid, fk, s);
+  else launch_lbm_t<T, 7>(P, mode, grid, fk, s);
 }
 
-int launch_lbm(const LbmParams& P0, int prec, int mode, cudaStream_t s) {
+int launch_lbm(const LbmParams& P0, int prec, int mode, const LbmFork& fk, cudaStream_t s) {
   LbmParams P = P0;
   const size_t esz = prec == PREC_FP32 ? sizeof(float) : sizeof(double);
   for (int q = 0; q < Q; ++q) {
@@ -1643,10 +1845,10 @@ int launch_lbm(const LbmParams& P0, int prec, int mode, cudaStream_t s) {
   }
   const long long threads = P.g.nwords * 32;
   const unsigned grid = (unsigned)((threads + LBM_THREADS - 1) / LBM_THREADS);
-  if (prec == PREC_FP32) launch_lbm_w<float>(P, mode, grid, s);
-  else if (prec == PREC_DF) launch_lbm_w<df>(P, mode, grid, s);
-  else launch_lbm_w<double>(P, mode, grid, s);
-  return 1;
+  if (prec == PREC_FP32) launch_lbm_w<float>(P, mode, grid, fk, s);
+  else if (prec == PREC_DF) launch_lbm_w<df>(P, mode, grid, fk, s);
+  else launch_lbm_w<double>(P, mode, grid, fk, s);
+  return prec == PREC_FP64 && P.mask ? 2 : 1;
 }
 
 static unsigned grid_for(long long n, int block) {
@@ -1732,15 +1934,20 @@ __device__ void fill_coef(CollideCoef<T>& c, const double* f, double wp, double 
   }
 }
 
-__global__ void step_const_kernel(MapParams P) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+__global__ void __launch_bounds__(FX_ROWS) step_const_kernel(MapParams P) {
   StepConst* sc = P.sc;
   const double vf = sc->vfluid;
   double f[3];
-  for (int a = 0; a < 3; ++a) {
+  for (int a = 0; a < 3; ++a)
     f[a] = P.fbody[a] - ((P.G[a] != 0.0 && vf > 0.0) ? P.G[a] / vf : 0.0);
-    sc->fext[a] = f[a];
+  // a thread per row of the fixed-point collision's table
+  if (P.fx_on) {
+    const int E0 = fx_e0(P.fx, f);
+    if (threadIdx.x == 0) sc->fx_E0 = E0;
+    if (E0 <= FX_EMAX) fx_row(P.fx, f, E0, threadIdx.x, sc->fx[threadIdx.x]);
   }
+  if (threadIdx.x != 0) return;
+  for (int a = 0; a < 3; ++a) sc->fext[a] = f[a];
   fill_coef<double>(sc->d, f, P.omega_p, P.omega_m);
   fill_coef<float>(sc->f, f, P.omega_p, P.omega_m);
   if (P.dfrec) fill_coef<df>(sc->x, f, P.omega_p, P.omega_m);
@@ -1752,7 +1959,7 @@ int launch_wait_selftest_lbm(unsigned* status, unsigned long long limit_ns, cuda
 }
 
 int launch_step_const(MapParams P, cudaStream_t s) {
-  step_const_kernel<<<1, 32, 0, s>>>(P);
+  step_const_kernel<<<1, FX_ROWS, 0, s>>>(P);
   return 1;
 }
 

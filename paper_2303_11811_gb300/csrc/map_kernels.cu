@@ -16,8 +16,7 @@
 //             3b. count8 counts them, four cells per warp;
 //   4. finish slots are ordered by particle index, MLP-mode and fallback cells
 //             get their eps, and B > 1 is normalised (every B_i divided by
-//             the sum); FP64 records: the mask of cells with one particle and
-//             B = 1.
+//             the sum).
 // Reach tests and sub-cell sampling take the FP64 definition's decisions: FP32
 // with a certified band and FP64 inside the band (geom.cuh); this file is
 // compiled with -fmad=false (fused multiply-adds only where written out).
@@ -1381,8 +1380,7 @@ __device__ __noinline__ WeightPair<T> pending_weights(const MapParams& P, int e,
 // pid and r0: the entry's particle pair and slot-0 record, loaded by the
 // caller a round ahead
 template <typename T, typename S>  // arithmetic in T, records stored as S
-__device__ double finish_entry(const MapParams& P, int e, int n, int2 pid, const T* pre,
-                               bool* full) {
+__device__ double finish_entry(const MapParams& P, int e, int n, int2 pid, const T* pre) {
   const bool live = e < n;
   T r0[4] = {pre[0], pre[1], pre[2], pre[3]}, r1[4] = {T(0), T(0), T(0), T(0)};
   S* V = static_cast<S*>(P.s.V);
@@ -1426,29 +1424,7 @@ __device__ double finish_entry(const MapParams& P, int e, int n, int2 pid, const
     P.s.pid[e] = pid;
     rec_store(V + 4 * e1, r1);
   }
-  *full = !two && r0[3] == T(1);
   return (double)B;
-}
-
-// the full-cell mask (one particle, B = 1: the FP64 collision takes these
-// cells in warps of their own, where the fluid change vanishes): the warp's
-// entries are consecutive slots, hence cells in increasing order; a
-// segmented OR over lanes of the same mask word leaves one atomicOr per run
-__device__ __forceinline__ void mark_full(const MapParams& P, int e, bool fl) {
-  const unsigned all = 0xffffffffu;
-  if (!__any_sync(all, fl)) return;
-  const int lane = threadIdx.x & 31;
-  const int cell = fl ? P.s.cell[e] : 0;
-  const int w = fl ? cell >> 5 : -1;
-  unsigned v = fl ? 1u << (cell & 31) : 0u;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const unsigned vu = __shfl_up_sync(all, v, off);
-    const int wu = __shfl_up_sync(all, w, off);
-    if (lane >= off && wu == w) v |= vu;
-  }
-  const int wn = __shfl_down_sync(all, w, 1);
-  if (fl && (lane == 31 || wn != w)) atomicOr(P.cov.full + w, v);
 }
 
 // one instance per record format (REC_*), so that each carries only its own
@@ -1483,9 +1459,7 @@ __global__ void __launch_bounds__(256, 3) finish_kernel(MapParams P) {
       pid_n = P.s.pid[e + stride];
       rec_load(V + 4 * (long long)(e + stride), rec_n);
     }
-    bool fl = false;
-    accB += finish_entry<T, S>(P, e, n, pid, r0, &fl);
-    if (REC == REC_FP64 && P.cov.full) mark_full(P, e, fl);
+    accB += finish_entry<T, S>(P, e, n, pid, r0);
   }
   red[threadIdx.x] = accB;
   __syncthreads();
@@ -1944,7 +1918,6 @@ int map_common(MapParams P, cudaStream_t s, bool mlp) {
   int launches = 0;
   cudaMemsetAsync(P.cov.mask, 0, sizeof(uint32_t) * P.g.nwords, s);
   cudaMemsetAsync(P.cov.dup, 0, sizeof(uint32_t) * P.g.nwords, s);
-  if (P.cov.full) cudaMemsetAsync(P.cov.full, 0, sizeof(uint32_t) * P.g.nwords, s);
   if (mlp) cudaMemsetAsync(P.mlp_count, 0, sizeof(int), s);
   if (P.p.n > 0) {
     box_kernel<<<(P.p.n + 127) / 128, 128, 0, s>>>(P);

@@ -38,11 +38,13 @@ struct psm_ctx {
   OpenBC bc{};         // constants of the open z faces
   bool open = false;   // an inflow or outflow face exists
   double tau = 0.6, omega_p = 0, omega_m = 0;
+  FxRates fx{};        // FP64 form: the fixed-point collision's relaxation constants
   int relax = 0, fp32 = 0, aa = 0;
   int prec = PREC_FP64;  // PDF storage and collision arithmetic (PREC_*)
   LbmPlan plan{};       // staged collision kernel (plan.stages = 0: not used)
   cudaStream_t stream = nullptr;
   cudaStream_t capture = nullptr;
+  LbmFork fork{};     // FP64: second stream of the collision
   std::vector<void*> allocs;
   void* buf[2] = {nullptr, nullptr};
   int cur = 0;        // pull: buffer holding f~ of the last step
@@ -69,6 +71,7 @@ struct psm_ctx {
   double* wtab = nullptr;        // B of the sampled counts (eps_n^3 < 513)
   bool have_wtab = false;
   unsigned* dem_bar = nullptr;   // grid barrier of the DEM step kernel
+  unsigned* work = nullptr;      // FP64 collision: counter of covered groups
   int dem_blocks = 0;            // resident blocks of the DEM step kernel
   float* mlp = nullptr;   // FP32 parameters on the device
   bool have_mlp = false;
@@ -203,6 +206,8 @@ MapParams map_params(psm_ctx* c) {
   }
   P.omega_p = c->omega_p;
   P.omega_m = c->omega_m;
+  P.fx = c->fx;
+  P.fx_on = c->prec == PREC_FP64;
   P.mlp = c->have_mlp ? c->mlp : nullptr;
   P.wtab = c->have_wtab ? c->wtab : nullptr;
   P.partials = c->partials;
@@ -261,7 +266,9 @@ int enqueue_step(psm_ctx* c, bool with_map, cudaStream_t s, bool dem = true) {
   if (c->p.n > 0) {
     L.mask = c->cov.mask;
     L.base = c->cov.base;
-    L.full = c->cov.full;
+    L.ncov = c->cov.ncov;
+    L.slot_cell = c->slots.cell;
+    L.work = c->work;
     L.slot_Fc = c->slots.Fc;
     L.slot_V = c->slots.V;
     L.slot_cap = c->slots.cap;
@@ -269,6 +276,7 @@ int enqueue_step(psm_ctx* c, bool with_map, cudaStream_t s, bool dem = true) {
   L.sc = c->sc;
   L.omega_p = c->omega_p;
   L.omega_m = c->omega_m;
+  L.fx = c->fx;
   L.bc = c->bc;
   L.status = c->status;
   L.tile_rows = c->plan.tile_rows;
@@ -276,10 +284,15 @@ int enqueue_step(psm_ctx* c, bool with_map, cudaStream_t s, bool dem = true) {
   L.stages = c->plan.stages;
   L.blocks = c->plan.blocks;
   L.smem = c->plan.smem;
+  L.nseg = c->plan.nseg;
+  L.seg_words = c->plan.seg_words;
+  L.div_words = c->plan.div_words;
+  L.div_seg = c->plan.div_seg;
+  L.cov_blocks = c->plan.cov_blocks;
   L.pf_ahead = c->plan.pf_ahead;
   {
     NvtxRange r("psm stream-collide");
-    n += launch_lbm(L, c->prec, mode, s);
+    n += launch_lbm(L, c->prec, mode, c->fork, s);
   }
   if (c->timing) cudaEventRecord(c->ev[2], s);
   if (c->p.n > 0) {
@@ -513,6 +526,7 @@ psm_status psm_create(const psm_grid* grid, double tau, psm_relax relax, const p
   c->stream = static_cast<cudaStream_t>(opt->stream);
   c->omega_p = 1.0 / tau;
   c->omega_m = relax == PSM_TRT ? 1.0 / (0.5 + opt->magic / (tau - 0.5)) : c->omega_p;
+  fx_fill(c->fx, c->omega_p, c->omega_m);
   c->log_e = opt->restitution > 0 ? std::log(opt->restitution) : 0.0;
   Grid& g = c->g;
   g.nx = grid->nx;
@@ -557,10 +571,6 @@ psm_status psm_create(const psm_grid* grid, double tau, psm_relax relax, const p
   c->cov.mask = alloc_n<uint32_t>(c, (size_t)g.nwords, c->allocs);
   c->cov.base = alloc_n<int>(c, (size_t)g.nwords, c->allocs);
   c->cov.dup = alloc_n<uint32_t>(c, (size_t)g.nwords, c->allocs);
-  if (c->prec == PREC_FP64) {
-    c->cov.full = alloc_n<uint32_t>(c, (size_t)g.nwords, c->allocs);
-    if (!c->cov.full) return bail(PSM_ERR_OOM, "allocator returned NULL");
-  }
   c->cov.nblocks = (g.nwords + 1023) / 1024;
   c->cov.blocksum = alloc_n<int>(c, (size_t)c->cov.nblocks, c->allocs);
   c->cov.ncov = alloc_n<int>(c, 1, c->allocs);
@@ -570,10 +580,12 @@ psm_status psm_create(const psm_grid* grid, double tau, psm_relax relax, const p
   c->mlp = alloc_n<float>(c, PSM_MLP_PARAMS, c->allocs);
   c->mlp_count = alloc_n<int>(c, 1, c->allocs);
   c->dem_bar = alloc_n<unsigned>(c, 4, c->allocs);
+  c->work = alloc_n<unsigned>(c, 1, c->allocs);
   // 513 doubles, 513 floats, 513 double-float pairs
   c->wtab = alloc_n<double>(c, 513 + 257 + 513, c->allocs);
   if (!c->cov.mask || !c->cov.base || !c->cov.dup || !c->cov.blocksum || !c->cov.ncov || !c->sc ||
-      !c->status || !c->partials || !c->mlp || !c->mlp_count || !c->dem_bar || !c->wtab)
+      !c->status || !c->partials || !c->mlp || !c->mlp_count || !c->dem_bar ||
+      !c->work || !c->wtab)
     return bail(PSM_ERR_OOM, "allocator returned NULL");
   cudaStream_t s = c->stream;
   bool ok = true;
@@ -581,10 +593,9 @@ psm_status psm_create(const psm_grid* grid, double tau, psm_relax relax, const p
     ok = ok && cudaMemsetAsync(c->buf[b], 0, esz * Q * (size_t)ncell, s) == cudaSuccess;
   ok = ok && cudaMemsetAsync(c->cov.mask, 0, sizeof(uint32_t) * g.nwords, s) == cudaSuccess;
   ok = ok && cudaMemsetAsync(c->cov.dup, 0, sizeof(uint32_t) * g.nwords, s) == cudaSuccess;
-  if (c->cov.full)
-    ok = ok && cudaMemsetAsync(c->cov.full, 0, sizeof(uint32_t) * g.nwords, s) == cudaSuccess;
   ok = ok && cudaMemsetAsync(c->status, 0, sizeof(unsigned), s) == cudaSuccess;
   ok = ok && cudaMemsetAsync(c->dem_bar, 0, 4 * sizeof(unsigned), s) == cudaSuccess;
+  ok = ok && cudaMemsetAsync(c->work, 0, sizeof(unsigned), s) == cudaSuccess;
   ok = ok && cudaMemsetAsync(c->cov.ncov, 0, sizeof(int), s) == cudaSuccess;
   StepConst h{};
   h.ncells = (double)g.nx * g.ny * g.nz;
@@ -615,6 +626,13 @@ psm_status psm_create(const psm_grid* grid, double tau, psm_relax relax, const p
   launch_step_const(map_params(c), s);
   c->have_wtab = launch_weight_table(c->opt.eps_n, c->tau, c->opt.weighting, c->wtab, s) > 0;
   if (cudaStreamCreateWithFlags(&c->capture, cudaStreamNonBlocking) != cudaSuccess) {
+    cudaGetLastError();
+    return bail(PSM_ERR_CUDA, "cudaStreamCreate failed");
+  }
+  if (c->prec == PREC_FP64 &&
+      (cudaStreamCreateWithFlags(&c->fork.side, cudaStreamNonBlocking) != cudaSuccess ||
+       cudaEventCreateWithFlags(&c->fork.fork, cudaEventDisableTiming) != cudaSuccess ||
+       cudaEventCreateWithFlags(&c->fork.join, cudaEventDisableTiming) != cudaSuccess)) {
     cudaGetLastError();
     return bail(PSM_ERR_CUDA, "cudaStreamCreate failed");
   }
@@ -1559,6 +1577,9 @@ void psm_destroy(psm_ctx* c) {
   for (auto& e : c->tev)
     if (e) cudaEventDestroy(e);
   if (c->capture) cudaStreamDestroy(c->capture);
+  if (c->fork.fork) cudaEventDestroy(c->fork.fork);
+  if (c->fork.join) cudaEventDestroy(c->fork.join);
+  if (c->fork.side) cudaStreamDestroy(c->fork.side);
   delete c;
 }
 

@@ -20,6 +20,7 @@
 #include <stdint.h>
 
 #include "df.cuh"
+#include "fixed64.cuh"
 
 namespace psm {
 
@@ -117,6 +118,10 @@ struct StepConst {
   CollideCoef<double> d;
   CollideCoef<float> f;
   CollideCoef<df> x;
+  // FP64 form: the fixed-point collision's smallest exponent and its table of
+  // forcing constants (fixed64.cuh)
+  FxRow fx[FX_ROWS];
+  int fx_E0;
 };
 
 struct Particles {
@@ -165,9 +170,6 @@ struct Slots {
 struct Coverage {
   uint32_t* mask;
   int* base;
-  // FP64 records only (else nullptr): bit = covered cell with one particle
-  // and B = 1 (every sample inside), written by the finish pass
-  uint32_t* full;
   // bit = cell in reach of two or more particles (the mark pass sets it when
   // its coverage bit was already set): a cell without it takes slot 0 with no
   // claim, and in surrogate mode it is the network's if partial
@@ -191,6 +193,8 @@ struct MapParams {
   double G[3];          // sum over free particles of (m - V) g
   double fbody[3];
   double omega_p, omega_m;
+  FxRates fx;           // FP64 form: relaxation constants of fixed64.cuh
+  int fx_on;
   const double* wtab;   // B of each sampled count c = 0..n^3 (n^3 < 513), or NULL;
                         // their FP32 roundings follow at (const float*)(wtab + 513)
   const float* mlp;     // FP32 parameters (PSM_MLP_PARAMS)
@@ -230,18 +234,27 @@ struct LbmParams {
   void* dstq[19];
   const uint32_t* mask; // nullptr when there are no particles
   const int* base;
-  const uint32_t* full; // Coverage::full (FP64 records), or nullptr
+  const int* ncov;      // number of covered cells (Coverage::ncov)
+  const int* slot_cell; // Slots::cell
+  unsigned* work;       // FP64: counter of the covered cells' groups
   void* slot_Fc;        // Slots::Fc
   const void* slot_V;   // Slots::V
   long long slot_cap;   // entries allocated
   const StepConst* sc;
   double omega_p, omega_m;
+  FxRates fx;           // FP64 form: relaxation constants of fixed64.cuh
   OpenBC bc;            // open z faces
   unsigned* status;     // device status word (ST_* bits)
   // staged kernel (stages > 0): tiles of tile_rows x-rows, `stages` tiles in
   // flight per block, `blocks` persistent blocks with `smem` bytes each
   int tile_rows, ntiles, stages, blocks;
   size_t smem;
+  // FP64: a row of more than 256 cells is staged in nseg segments of
+  // seg_words coverage words, a tile each; divisions by a tile's words and by
+  // the segments of a row
+  int nseg, seg_words;
+  FastDiv div_words, div_seg;
+  int cov_blocks;       // blocks of the kernel of the covered cells
   // one-cell-per-thread FP32 pull kernel: each block prefetches into L2 the
   // source spans of the block pf_ahead places later (0: no prefetch)
   int pf_ahead;
@@ -250,6 +263,9 @@ struct LbmParams {
 struct LbmPlan {
   int tile_rows, ntiles, stages, blocks;
   size_t smem;
+  int nseg, seg_words;
+  FastDiv div_words, div_seg;
+  int cov_blocks;
   int pf_ahead;
 };
 
@@ -257,7 +273,13 @@ struct LbmPlan {
 int lbm_configure();  // kernel attributes; call once before launching (returns != 0 on error)
 // staged-kernel plan for a grid (stages = 0: use the one-cell-per-thread kernel)
 int lbm_plan(const Grid& g, int prec, int aa, LbmPlan* plan);
-int launch_lbm(const LbmParams& P, int prec, int mode, cudaStream_t s);
+// FP64: the covered cells' kernel runs beside the other on a second stream,
+// which forks from s and joins it again (side = nullptr: one after the other)
+struct LbmFork {
+  cudaStream_t side;
+  cudaEvent_t fork, join;
+};
+int launch_lbm(const LbmParams& P, int prec, int mode, const LbmFork& fk, cudaStream_t s);
 // a box of cells, origin (x0, y0, z0) (non-negative, taken modulo the grid) and
 // extent (bx, by, bz); output layout [q][z][y][x] over the box
 struct BoxSel {
