@@ -100,98 +100,259 @@ __global__ void samples_kernel(unsigned long long seed, long long first, long lo
   }
 }
 
-// ---- training: forward + backward of one tile of samples
+// ---- training: forward + backward of one tile of samples.  A tile is 128
+// samples, 8 to each of the block's 16 warps: a thread computes 4 samples x 2
+// units of a layer, reading inputs and weights four at a time along the sum
+// (rows of 36 floats: eight rows' 16-byte pieces fall in different banks), and
+// only the warp itself meets between layers.  Every sum runs in a fixed order
+// (a unit's over its inputs, a gradient's over the tile's samples), so the
+// result does not depend on how the work is split.  One thread per sample, as
+// before, left 4 warps an SM to two shared-memory reads per multiply-add.
 constexpr int TILE = 128;
-constexpr int ROW = 33;  // padded row of 32 activations (bank-conflict free)
+constexpr int ROW = 36;
+constexpr int TRAIN_THREADS = 512;
+static_assert(TRAIN_THREADS == 4 * TILE, "8 samples per warp");
 
+// the network's parameters as the layers read them (W2 also transposed, for
+// the backward product)
+struct alignas(16) NetSmem {
+  float w1[32][4];
+  float b1[32];
+  float w2[32][ROW];
+  float w2t[32][ROW];
+  float b2[32], w3[32];
+  float b3, one;
+};
+// places (in floats) of packed parameter e
+__device__ __forceinline__ int net_place(int e, int* second) {
+  constexpr int B1 = 128, W2 = 160, W2T = W2 + 32 * ROW, B2 = W2T + 32 * ROW;
+  *second = -1;
+  if (e < OFF_W2) return e;  // w1, b1
+  if (e < OFF_B2) {
+    const int j = (e - OFF_W2) >> 5, k = (e - OFF_W2) & 31;
+    *second = W2T + k * ROW + j;
+    return W2 + j * ROW + k;
+  }
+  static_assert(OFF_B1 == B1 && OFF_W2 == W2 && OFF_W3 == OFF_B2 + 32 && OFF_B3 == OFF_W3 + 32,
+                "b2, w3 and b3 follow one another");
+  return B2 + (e - OFF_B2);
+}
 struct TrainSmem {
-  float p[NPARAM + 3];
-  float x[TILE][4];
-  float h1[TILE][ROW];
-  float h2[TILE][ROW];
-  float dh1[TILE][ROW];
-  float dh2[TILE][ROW];
-  float dy[TILE];
-  float l2[TILE];
+  NetSmem net;
+  float4 x[TILE];
+  float h1[TILE][ROW], h2[TILE][ROW];    // activations
+  float dh1[TILE][ROW], dh2[TILE][ROW];  // gradients before the ReLU
+  float4 dyl[TILE];                      // d loss / d y, squared residual
 };
 
-__global__ void __launch_bounds__(TILE) train_tile_kernel(const float* __restrict__ params,
-                                                         long long m,
-                                                         const float* __restrict__ X,
-                                                         const float* __restrict__ t,
-                                                         float* __restrict__ partials) {
+__device__ __forceinline__ void load_net(TrainSmem& S, const float* __restrict__ params) {
+  float* n = reinterpret_cast<float*>(&S.net);
+  for (int e = threadIdx.x; e < NPARAM; e += TRAIN_THREADS) {
+    int b;
+    const int a = net_place(e, &b);
+    const float v = params[e];
+    n[a] = v;
+    if (b >= 0) n[b] = v;
+  }
+  if (threadIdx.x == 0) S.net.one = 1.0f;
+}
+
+// a lane's input of a tile: lanes 0-7 of warp w hold samples 8w .. 8w + 7
+struct SampleIn {
+  float x[4], t;
+};
+__device__ __forceinline__ void load_sample(const float* __restrict__ X,
+                                            const float* __restrict__ t, long long first,
+                                            int nrow, SampleIn& I) {
+  const int s = 8 * (threadIdx.x >> 5) + (threadIdx.x & 31);
+  const bool in = (threadIdx.x & 31) < 8 && s < nrow;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) I.x[k] = in ? X[4 * (first + s) + k] : 0.f;
+  I.t = in ? t[first + s] : 0.f;
+}
+
+__device__ __forceinline__ float4 row4(const float* row, int c) {
+  return reinterpret_cast<const float4*>(row)[c];
+}
+__device__ __forceinline__ float chain4(float acc, const float4& w, const float4& v) {
+  acc = fmaf(w.x, v.x, acc);
+  acc = fmaf(w.y, v.y, acc);
+  acc = fmaf(w.z, v.z, acc);
+  return fmaf(w.w, v.w, acc);
+}
+
+// forward (and backward) of the warp's 8 samples; rows nrow and up count as zeros
+template <bool BACK>
+__device__ __forceinline__ void tile_rows(TrainSmem& S, int nrow, const SampleIn& I,
+                                          float inv_m) {
+  const int lane = threadIdx.x & 31, s0 = 8 * (threadIdx.x >> 5);
+  const int sb = s0 + 4 * (lane >> 4), jg = lane & 15;  // samples sb .. sb + 3, units jg, jg + 16
+  if (lane < 8) S.x[s0 + lane] = make_float4(I.x[0], I.x[1], I.x[2], I.x[3]);
+  __syncwarp();
+  float h1[4][2], h2[4][2];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int j = jg + 16 * i;
+    const float4 w = row4(S.net.w1[j], 0);
+    const float b = S.net.b1[j];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const float a = chain4(b, w, S.x[sb + r]);
+      h1[r][i] = a > 0.f && sb + r < nrow ? a : 0.f;
+      S.h1[sb + r][j] = h1[r][i];
+    }
+  }
+  __syncwarp();
+  float acc[4][2];
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int i = 0; i < 2; ++i) acc[r][i] = S.net.b2[jg + 16 * i];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const float4 wa = row4(S.net.w2[jg], c), wb = row4(S.net.w2[jg + 16], c);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const float4 h = row4(S.h1[sb + r], c);
+      acc[r][0] = chain4(acc[r][0], wa, h);
+      acc[r][1] = chain4(acc[r][1], wb, h);
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      h2[r][i] = acc[r][i] > 0.f && sb + r < nrow ? acc[r][i] : 0.f;
+      S.h2[sb + r][jg + 16 * i] = h2[r][i];
+    }
+  __syncwarp();
+  if (lane < 8) {
+    float y = S.net.b3;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) y = chain4(y, row4(S.net.w3, c), row4(S.h2[s0 + lane], c));
+    const float res = y - I.t;
+    const float dy = 2.0f * res * inv_m;
+    S.dyl[s0 + lane] = s0 + lane < nrow ? make_float4(dy, res * res, 0.f, 0.f)
+                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  if constexpr (BACK) {
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const float dy = S.dyl[sb + r].x;
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        S.dh2[sb + r][jg + 16 * i] = h2[r][i] > 0.f ? dy * S.net.w3[jg + 16 * i] : 0.f;
+        acc[r][i] = 0.f;
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const float4 wa = row4(S.net.w2t[jg], c), wb = row4(S.net.w2t[jg + 16], c);
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const float4 d = row4(S.dh2[sb + r], c);
+        acc[r][0] = chain4(acc[r][0], wa, d);
+        acc[r][1] = chain4(acc[r][1], wb, d);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+        S.dh1[sb + r][jg + 16 * i] = h1[r][i] > 0.f ? acc[r][i] : 0.f;
+  }
+}
+
+// gradient of the tile (sums over its samples in order) and its squared
+// residual: four warps take dW2, 4 x 2 entries per thread, two the rest (the
+// biases' sums as products with one)
+__device__ __forceinline__ void tile_grad(const TrainSmem& S, float* __restrict__ out) {
+  const int warp = threadIdx.x >> 5;
+  if (warp < 4) {
+    const int jg = threadIdx.x & 7, kg = threadIdx.x >> 3;  // rows 4 jg .., columns 2 kg ..
+    float g[4][2] = {};
+#pragma unroll 8
+    for (int q = 0; q < TILE; ++q) {
+      const float4 d = row4(S.dh2[q], jg);
+      const float2 h = reinterpret_cast<const float2*>(S.h1[q])[kg];
+      g[0][0] = fmaf(d.x, h.x, g[0][0]);
+      g[0][1] = fmaf(d.x, h.y, g[0][1]);
+      g[1][0] = fmaf(d.y, h.x, g[1][0]);
+      g[1][1] = fmaf(d.y, h.y, g[1][1]);
+      g[2][0] = fmaf(d.z, h.x, g[2][0]);
+      g[2][1] = fmaf(d.z, h.y, g[2][1]);
+      g[3][0] = fmaf(d.w, h.x, g[3][0]);
+      g[3][1] = fmaf(d.w, h.y, g[3][1]);
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      out[OFF_W2 + (4 * jg + c) * 32 + 2 * kg] = g[c][0];
+      out[OFF_W2 + (4 * jg + c) * 32 + 2 * kg + 1] = g[c][1];
+    }
+  } else if (warp < 6) {
+    const int it = threadIdx.x - 128, jg = it & 7;
+    const float* v;         // four values per sample, rows of vs floats
+    const float* a = &S.net.one;  // their factor, as floats apart
+    int vs = ROW, as = 0, o, os = 1, n = 4;
+    if (it < 32) {  // dW1
+      v = S.dh1[0] + 4 * jg;
+      a = reinterpret_cast<const float*>(S.x) + (it >> 3);
+      as = 4;
+      o = 16 * jg + (it >> 3);
+      os = 4;
+    } else if (it < 40) {
+      v = S.dh1[0] + 4 * jg;
+      o = OFF_B1 + 4 * jg;
+    } else if (it < 48) {
+      v = S.dh2[0] + 4 * jg;
+      o = OFF_B2 + 4 * jg;
+    } else if (it < 56) {
+      v = S.h2[0] + 4 * jg;
+      a = &S.dyl[0].x;
+      as = 4;
+      o = OFF_W3 + 4 * jg;
+    } else {  // db3 and the loss
+      v = &S.dyl[0].x;
+      vs = 4;
+      o = OFF_B3;
+      n = it == 56 ? 2 : 0;
+    }
+    float g[4] = {};
+#pragma unroll 8
+    for (int q = 0; q < TILE; ++q) {
+      const float4 d = row4(v + q * vs, 0);
+      const float f = a[q * as];
+      g[0] = fmaf(d.x, f, g[0]);
+      g[1] = fmaf(d.y, f, g[1]);
+      g[2] = fmaf(d.z, f, g[2]);
+      g[3] = fmaf(d.w, f, g[3]);
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      if (c < n) out[o + c * os] = g[c];
+  }
+}
+
+__device__ __forceinline__ int tile_count(long long m, long long first) {
+  return (int)(m - first < TILE ? m - first : TILE);
+}
+
+__global__ void __launch_bounds__(TRAIN_THREADS) train_tile_kernel(
+    const float* __restrict__ params, long long m, const float* __restrict__ X,
+    const float* __restrict__ t, float* __restrict__ partials) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TrainSmem& S = *reinterpret_cast<TrainSmem*>(smem_raw);
-  for (int i = threadIdx.x; i < NPARAM; i += TILE) S.p[i] = params[i];
+  const long long first = (long long)blockIdx.x * TILE;
+  const int nrow = tile_count(m, first);
+  SampleIn I;
+  load_sample(X, t, first, nrow, I);
+  load_net(S, params);
   __syncthreads();
-  const long long s = (long long)blockIdx.x * TILE + threadIdx.x;
-  const int r = threadIdx.x;
-  const float inv_m = 1.0f / (float)m;
-  if (s < m) {
-    float x[4];
-    for (int k = 0; k < 4; ++k) x[k] = X[4 * s + k];
-    float a1[32], h2v[32];
-    for (int j = 0; j < 32; ++j) {
-      float acc = S.p[OFF_B1 + j];
-      for (int k = 0; k < 4; ++k) acc = fmaf(S.p[j * 4 + k], x[k], acc);
-      a1[j] = acc;
-      S.h1[r][j] = acc > 0.f ? acc : 0.f;
-    }
-    float y = S.p[OFF_B3];
-    for (int j = 0; j < 32; ++j) {
-      float acc = S.p[OFF_B2 + j];
-      for (int k = 0; k < 32; ++k) acc = fmaf(S.p[OFF_W2 + j * 32 + k], S.h1[r][k], acc);
-      h2v[j] = acc;  // pre-activation
-      const float h = acc > 0.f ? acc : 0.f;
-      S.h2[r][j] = h;
-      y = fmaf(S.p[OFF_W3 + j], h, y);
-    }
-    const float res = y - t[s];
-    const float dy = 2.0f * res * inv_m;
-    S.dy[r] = dy;
-    S.l2[r] = res * res;
-    for (int j = 0; j < 32; ++j) S.dh2[r][j] = h2v[j] > 0.f ? dy * S.p[OFF_W3 + j] : 0.f;
-    for (int k = 0; k < 32; ++k) {
-      float acc = 0.f;
-      for (int j = 0; j < 32; ++j) acc = fmaf(S.p[OFF_W2 + j * 32 + k], S.dh2[r][j], acc);
-      S.dh1[r][k] = a1[k] > 0.f ? acc : 0.f;
-    }
-    for (int k = 0; k < 4; ++k) S.x[r][k] = x[k];
-  } else {
-    for (int j = 0; j < 32; ++j) {
-      S.h1[r][j] = 0.f; S.h2[r][j] = 0.f; S.dh1[r][j] = 0.f; S.dh2[r][j] = 0.f;
-    }
-    for (int k = 0; k < 4; ++k) S.x[r][k] = 0.f;
-    S.dy[r] = 0.f;
-    S.l2[r] = 0.f;
-  }
+  tile_rows<true>(S, nrow, I, 1.0f / (float)m);
   __syncthreads();
-  // gradient of this tile: sums over its samples in a fixed order
-  float* out = partials + (long long)blockIdx.x * (NPARAM + 1);
-  for (int e = threadIdx.x; e < NPARAM + 1; e += TILE) {
-    float acc = 0.f;
-    if (e < OFF_B1) {  // dW1[j][k]
-      const int j = e / 4, k = e % 4;
-      for (int q = 0; q < TILE; ++q) acc = fmaf(S.dh1[q][j], S.x[q][k], acc);
-    } else if (e < OFF_W2) {  // db1
-      const int j = e - OFF_B1;
-      for (int q = 0; q < TILE; ++q) acc += S.dh1[q][j];
-    } else if (e < OFF_B2) {  // dW2[j][k]
-      const int j = (e - OFF_W2) / 32, k = (e - OFF_W2) % 32;
-      for (int q = 0; q < TILE; ++q) acc = fmaf(S.dh2[q][j], S.h1[q][k], acc);
-    } else if (e < OFF_W3) {  // db2
-      const int j = e - OFF_B2;
-      for (int q = 0; q < TILE; ++q) acc += S.dh2[q][j];
-    } else if (e < OFF_B3) {  // dW3
-      const int j = e - OFF_W3;
-      for (int q = 0; q < TILE; ++q) acc = fmaf(S.dy[q], S.h2[q][j], acc);
-    } else if (e == OFF_B3) {
-      for (int q = 0; q < TILE; ++q) acc += S.dy[q];
-    } else {  // loss numerator
-      for (int q = 0; q < TILE; ++q) acc += S.l2[q];
-    }
-    out[e] = acc;
-  }
+  tile_grad(S, partials + (long long)blockIdx.x * (NPARAM + 1));
 }
 
 __global__ void grad_reduce_kernel(const float* __restrict__ partials, int nblocks,
@@ -205,18 +366,141 @@ __global__ void grad_reduce_kernel(const float* __restrict__ partials, int nbloc
   else if (loss) *loss = acc * inv_m;
 }
 
+// one parameter's Adam step
+__device__ __forceinline__ void adam(float gi, const AdamStep& a, float& p, float& m, float& v) {
+  const float mi = 0.9f * m + 0.1f * gi;
+  const float vi = 0.999f * v + 0.001f * gi * gi;
+  m = mi;
+  v = vi;
+  const float mh = mi / a.bc1, vh = vi / a.bc2;
+  p -= a.lr * mh / (sqrtf(vh) + 1e-8f);
+}
+
 __global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g,
-                            float* __restrict__ m, float* __restrict__ v, float bc1, float bc2,
-                            float lr) {
+                            float* __restrict__ m, float* __restrict__ v, AdamStep a) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= NPARAM) return;
-  const float gi = g[i];
-  const float mi = 0.9f * m[i] + 0.1f * gi;
-  const float vi = 0.999f * v[i] + 0.001f * gi * gi;
-  m[i] = mi;
-  v[i] = vi;
-  const float mh = mi / bc1, vh = vi / bc2;
-  p[i] -= lr * mh / (sqrtf(vh) + 1e-8f);
+  if (i < NPARAM) adam(g[i], a, p[i], m[i], v[i]);
+}
+
+// ---- minibatch steps one after another in one launch: a cluster of 8 CTAs
+// keeps the network in shared memory.  Per step the CTAs take the
+// minibatch's tiles in turn and leave their gradients in `partials`; each CTA
+// sums an eighth of the entries over the tiles in order, applies Adam (its
+// moments stay in registers) and writes the new values into every CTA's copy.
+// Two cluster barriers per step stand for the three launches they replace.
+// Bound by latency: of the 8.8 us of a minibatch of 1024 samples most is the
+// chain of layers, gradient sums, barriers and the sum over the tiles (a tile's
+// multiply-adds alone would take 2 us of its SM).  Before, with one thread per
+// sample and three launches, 35 us.
+constexpr int CLUSTER = 8;
+constexpr int SLICE = (NPARAM + CLUSTER - 1) / CLUSTER;
+
+__device__ __forceinline__ void cluster_sync_all() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void store_cluster(const float* local, unsigned rank, float v) {
+  unsigned a = (unsigned)__cvta_generic_to_shared(local), r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(r), "f"(v) : "memory");
+}
+
+// minibatch i of the launch: samples b0 + i batch (mod nsamples' minibatches,
+// per_epoch of them) ..; sched[i]: its Adam coefficients
+__global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(TRAIN_THREADS, 1)
+    train_cluster_kernel(float* __restrict__ params, float* __restrict__ mstate,
+                         float* __restrict__ vstate, const float* __restrict__ X,
+                         const float* __restrict__ t, long long nsamples, int batch,
+                         long long per_epoch, long long mb0, int steps,
+                         const AdamStep* __restrict__ sched, float* __restrict__ partials) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  TrainSmem& S = *reinterpret_cast<TrainSmem*>(smem_raw);
+  const int rank = (int)blockIdx.x;  // the grid is one cluster
+  const int e = rank * SLICE + (int)threadIdx.x;
+  const bool own = threadIdx.x < SLICE && e < NPARAM;
+  int pb = -1;
+  const int pa = own ? net_place(e, &pb) : 0;
+  float p = 0.f, mo = 0.f, ve = 0.f;
+  if (own) {
+    p = params[e];
+    mo = mstate[e];
+    ve = vstate[e];
+  }
+  load_net(S, params);
+  cluster_sync_all();  // every CTA runs before its shared memory is written
+  long long mb = mb0;
+  SampleIn I;
+  auto load_first = [&](long long b) {  // the CTA's first tile of minibatch b
+    const long long s = b * batch, n = min((long long)batch, nsamples - s);
+    const long long first = (long long)rank * TILE;
+    load_sample(X, t, s + first, first < n ? tile_count(n, first) : 0, I);
+  };
+  load_first(mb);
+  for (int i = 0; i < steps; ++i) {
+    const long long s = mb * batch;
+    const int n = (int)min((long long)batch, nsamples - s);
+    const int ntile = (n + TILE - 1) / TILE;
+    const float inv_m = 1.0f / (float)(long long)n;
+    const AdamStep a = sched[i];
+    for (int k = rank; k < ntile; k += CLUSTER) {
+      const int nrow = tile_count(n, (long long)k * TILE);
+      if (k != rank) {
+        load_sample(X, t, s + (long long)k * TILE, nrow, I);
+        __syncthreads();  // the previous tile's gradient is done
+      }
+      tile_rows<true>(S, nrow, I, inv_m);
+      __syncthreads();
+      tile_grad(S, partials + (long long)k * (NPARAM + 1));
+    }
+    mb = mb + 1 == per_epoch ? 0 : mb + 1;
+    if (i + 1 < steps) load_first(mb);  // on its way while the CTAs meet
+    cluster_sync_all();
+    if (own) {
+      float g = 0.f;
+#pragma unroll 8
+      for (int k = 0; k < ntile; ++k) g += __ldcg(partials + (long long)k * (NPARAM + 1) + e);
+      adam(g, a, p, mo, ve);
+      const float* net = reinterpret_cast<const float*>(&S.net);
+#pragma unroll
+      for (unsigned r = 0; r < CLUSTER; ++r) {
+        store_cluster(net + pa, r, p);
+        if (pb >= 0) store_cluster(net + pb, r, p);
+      }
+    }
+    cluster_sync_all();
+  }
+  if (own) {
+    params[e] = p;
+    mstate[e] = mo;
+    vstate[e] = ve;
+  }
+}
+
+// squared residuals of each minibatch's tiles (tiles per minibatch, the
+// last one's may be fewer)
+__global__ void __launch_bounds__(TRAIN_THREADS) train_loss_kernel(
+    const float* __restrict__ params, const float* __restrict__ X, const float* __restrict__ t,
+    long long nsamples, int batch, int tiles, long long ntiles, float* __restrict__ out) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  TrainSmem& S = *reinterpret_cast<TrainSmem*>(smem_raw);
+  load_net(S, params);
+  for (long long w = blockIdx.x; w < ntiles; w += gridDim.x) {
+    const long long mb = w / tiles, first = (w - mb * tiles) * TILE, s = mb * batch;
+    const long long n = min((long long)batch, nsamples - s);
+    const int nrow = first < n ? tile_count(n, first) : 0;
+    SampleIn I;
+    load_sample(X, t, s + first, nrow, I);
+    __syncthreads();  // the network; the previous tile's sum is done
+    tile_rows<false>(S, nrow, I, 0.f);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      float acc = 0.f;
+#pragma unroll 8
+      for (int q = 0; q < TILE; ++q) acc += S.dyl[q].y;
+      out[w] = acc;
+    }
+  }
 }
 
 // ---- inference on the 5th-generation tensor cores.  One CTA of 128
@@ -563,24 +847,61 @@ int mlp_grad_blocks(long long m) { return (int)((m + TILE - 1) / TILE); }
 int launch_mlp_loss_grad(const float* params, long long m, const float* X, const float* t,
                          float* grad_partials, int nblocks, float* grad, float* loss,
                          cudaStream_t s) {
-  static bool configured = false;
-  const int smem = (int)sizeof(TrainSmem);
-  if (!configured) {
-    cudaFuncSetAttribute(train_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    configured = true;
-  }
-  train_tile_kernel<<<nblocks, TILE, smem, s>>>(params, m, X, t, grad_partials);
+  train_tile_kernel<<<nblocks, TRAIN_THREADS, sizeof(TrainSmem), s>>>(params, m, X, t,
+                                                                      grad_partials);
   grad_reduce_kernel<<<(NPARAM + 1 + 255) / 256, 256, 0, s>>>(grad_partials, nblocks, grad,
                                                              loss, 1.0f / (float)m);
   return 2;
 }
 
-int launch_adam(float* params, const float* grad, float* mstate, float* vstate, int step,
-                float lr, cudaStream_t s) {
-  const float bc1 = 1.0f - powf(0.9f, (float)step);
-  const float bc2 = 1.0f - powf(0.999f, (float)step);
-  adam_kernel<<<(NPARAM + 255) / 256, 256, 0, s>>>(params, grad, mstate, vstate, bc1, bc2, lr);
+// Minibatches of up to kClusterTiles tiles train in the cluster kernel, all
+// `steps` in one launch; larger ones, whose tiles fill more SMs than a cluster
+// has, in three launches each.  Per minibatch of 8, 16, 32 and 64 tiles the
+// cluster kernel takes 8.8, 14.8, 26.8 and 51 us, the launches 18.4 each.
+constexpr int kClusterTiles = 16;
+int launch_train_steps(float* params, float* mstate, float* vstate, const float* X, const float* t,
+                       long long nsamples, int batch, long long per_epoch, long long mb0,
+                       int steps, const AdamStep* sched_host, AdamStep* sched, float* partials,
+                       float* grad, cudaStream_t s) {
+  const int tiles = mlp_grad_blocks(batch < nsamples ? batch : nsamples);
+  if (tiles <= kClusterTiles) {
+    cudaMemcpyAsync(sched, sched_host, sizeof(AdamStep) * steps, cudaMemcpyHostToDevice, s);
+    train_cluster_kernel<<<CLUSTER, TRAIN_THREADS, sizeof(TrainSmem), s>>>(
+        params, mstate, vstate, X, t, nsamples, batch, per_epoch, mb0, steps, sched, partials);
+    return 1;
+  }
+  for (int i = 0; i < steps; ++i) {
+    const long long b0 = (mb0 + i) % per_epoch * batch;
+    const long long m = nsamples - b0 < batch ? nsamples - b0 : batch;
+    launch_mlp_loss_grad(params, m, X + 4 * b0, t + b0, partials, mlp_grad_blocks(m), grad,
+                         nullptr, s);
+    adam_kernel<<<(NPARAM + 255) / 256, 256, 0, s>>>(params, grad, mstate, vstate, sched_host[i]);
+  }
+  return 3 * steps;
+}
+
+long long train_loss_tiles(long long nsamples, int batch) {
+  const long long b = batch < nsamples ? batch : nsamples;
+  return (nsamples + b - 1) / b * mlp_grad_blocks(b);
+}
+
+int launch_train_loss(const float* params, const float* X, const float* t, long long nsamples,
+                      int batch, float* out, cudaStream_t s) {
+  const long long n = train_loss_tiles(nsamples, batch);
+  const int tiles = mlp_grad_blocks(batch < nsamples ? batch : nsamples);
+  const long long blocks = n < 152 * 2 ? n : 152 * 2;
+  train_loss_kernel<<<(unsigned)blocks, TRAIN_THREADS, sizeof(TrainSmem), s>>>(
+      params, X, t, nsamples, batch, tiles, n, out);
   return 1;
+}
+
+int mlp_train_configure() {
+  const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  const int smem = (int)sizeof(TrainSmem);
+  int bad = cudaFuncSetAttribute(train_tile_kernel, a, smem) != cudaSuccess;
+  bad |= cudaFuncSetAttribute(train_cluster_kernel, a, smem) != cudaSuccess;
+  bad |= cudaFuncSetAttribute(train_loss_kernel, a, smem) != cudaSuccess;
+  return bad;
 }
 
 int launch_wait_selftest_mlp(unsigned* status, unsigned long long limit_ns, cudaStream_t s) {

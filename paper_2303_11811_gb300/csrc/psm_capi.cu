@@ -610,7 +610,7 @@ psm_status psm_create(const psm_grid* grid, double tau, psm_relax relax, const p
     cudaGetLastError();
     return bail(PSM_ERR_CUDA, "could not set the shared-memory size of the collision kernel");
   }
-  if (mlp_configure() != 0) {
+  if (mlp_configure() != 0 || mlp_train_configure() != 0) {
     cudaGetLastError();
     return bail(PSM_ERR_CUDA, "occupancy query of the inference kernel failed");
   }
@@ -1315,48 +1315,68 @@ psm_status psm_mlp_infer(psm_ctx* c, const float* params, long m, const float* X
   return PSM_OK;
 }
 
+// minibatches per launch of the training kernel (9 ms at 1024 samples each)
+static constexpr int kTrainChunk = 1024;
+
 psm_status psm_train_surrogate(psm_ctx* c, long nsamples, unsigned long long seed, int epochs,
                                int batch, float lr, float* loss_out) {
   if (!c || nsamples <= 0 || epochs < 1 || batch < 1 || !(lr > 0)) return PSM_ERR_ARG;
   if (!c->have_mlp) return fail(c, PSM_ERR_STATE, "set initial surrogate parameters first");
+  const long per_epoch = (nsamples + batch - 1) / batch;
+  const long long steps = (long long)per_epoch * epochs;
+  const long long nt = train_loss_tiles(nsamples, batch);
+  std::vector<AdamStep> sh;  // a chunk's Adam steps
+  std::vector<float> tl;     // tiles' losses
+  try {
+    sh.resize((size_t)std::min<long long>(steps, kTrainChunk));
+    tl.resize((size_t)nt);
+  } catch (...) {
+    return fail(c, PSM_ERR_OOM, "out of host memory");
+  }
   const int nb = mlp_grad_blocks(batch);
   const size_t floats = 6 * (size_t)nsamples + 3 * PSM_MLP_PARAMS + 1 +
-                        (size_t)nb * (PSM_MLP_PARAMS + 1);
+                        (size_t)nb * (PSM_MLP_PARAMS + 1) +
+                        sizeof(AdamStep) / sizeof(float) * kTrainChunk;
   float* d = static_cast<float*>(dalloc(c, sizeof(float) * floats));
   if (!d) return fail(c, PSM_ERR_OOM, "allocator returned NULL");
   float* X = d;
   float* T = X + 4 * nsamples;   // residual targets: label - eps_lin
-  float* L = T + nsamples;       // labels (unused by the optimiser)
+  float* L = T + nsamples;       // labels (unused by the optimiser); the tiles' losses at the end
   float* g = L + nsamples;
   float* ms = g + PSM_MLP_PARAMS;
   float* vs = ms + PSM_MLP_PARAMS;
-  float* dl = vs + PSM_MLP_PARAMS;
-  float* part = dl + 1;
+  AdamStep* sched = reinterpret_cast<AdamStep*>(vs + PSM_MLP_PARAMS);
+  float* part = reinterpret_cast<float*>(sched + kTrainChunk);
   cudaStream_t s = c->stream;
   launch_mlp_samples(seed, 0, nsamples, X, L, T, s);
   cudaMemsetAsync(ms, 0, sizeof(float) * 2 * PSM_MLP_PARAMS, s);
-  int step = 0;
   double last = 0.0;
-  const long per_epoch = (nsamples + batch - 1) / batch;
   const double total = (double)per_epoch * epochs;
-  for (int ep = 0; ep < epochs; ++ep) {
-    for (long b0 = 0; b0 < nsamples; b0 += batch) {
-      const long mb = nsamples - b0 < batch ? nsamples - b0 : batch;
-      launch_mlp_loss_grad(c->mlp, mb, X + 4 * b0, T + b0, part, mlp_grad_blocks(mb), g, dl, s);
+  for (long long step = 0; step < steps;) {
+    const int k = (int)std::min<long long>(steps - step, kTrainChunk);
+    const long long first = step;
+    for (int i = 0; i < k; ++i) {
       // learning rate decays exponentially to 3% of lr over the run
-      const float lr_t = (float)(lr * std::pow(0.03, (double)step / total));
-      launch_adam(c->mlp, g, ms, vs, ++step, lr_t, s);
+      sh[i].lr = (float)(lr * std::pow(0.03, (double)step / total));
+      ++step;
+      sh[i].bc1 = 1.0f - powf(0.9f, (float)step);
+      sh[i].bc2 = 1.0f - powf(0.999f, (float)step);
     }
+    launch_train_steps(c->mlp, ms, vs, X, T, nsamples, batch, per_epoch, first % per_epoch, k,
+                       sh.data(), sched, part, g, s);
   }
   // loss of the final parameters over the whole sample set, in minibatches
+  launch_train_loss(c->mlp, X, T, nsamples, batch, L, s);
+  cudaMemcpyAsync(tl.data(), L, sizeof(float) * nt, cudaMemcpyDeviceToHost, s);
   double acc = 0.0;
-  for (long b0 = 0; b0 < nsamples; b0 += batch) {
-    const long mb = nsamples - b0 < batch ? nsamples - b0 : batch;
-    launch_mlp_loss_grad(c->mlp, mb, X + 4 * b0, T + b0, part, mlp_grad_blocks(mb), g, dl, s);
-    float hl = 0;
-    cudaMemcpyAsync(&hl, dl, sizeof(float), cudaMemcpyDeviceToHost, s);
-    if (cudaStreamSynchronize(s) != cudaSuccess) break;
-    acc += (double)hl * mb;
+  if (cudaStreamSynchronize(s) == cudaSuccess) {
+    const long long tiles = nt / per_epoch;
+    for (long b = 0; b < per_epoch; ++b) {
+      const long mb = std::min<long>(batch, nsamples - b * batch);
+      float hl = 0.f;
+      for (int k = 0; k < mlp_grad_blocks(mb); ++k) hl += tl[b * tiles + k];
+      acc += (double)(hl * (1.0f / (float)mb)) * mb;
+    }
   }
   last = acc / nsamples;
   cudaError_t e = cudaGetLastError();

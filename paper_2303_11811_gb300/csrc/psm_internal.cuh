@@ -349,8 +349,23 @@ int launch_mlp_samples(unsigned long long seed, long long first, long long count
 int launch_mlp_loss_grad(const float* params, long long m, const float* X, const float* t,
                          float* grad_partials, int nblocks, float* grad, float* loss,
                          cudaStream_t s);
-int launch_adam(float* params, const float* grad, float* mstate, float* vstate, int step,
-                float lr, cudaStream_t s);
+// bias corrections 1 - 0.9^k, 1 - 0.999^k and learning rate of Adam step k
+struct AdamStep {
+  float bc1, bc2, lr;
+};
+// `steps` minibatches from minibatch mb0 on (sched_host: their Adam steps;
+// sched: room for as many on the device; partials: mlp_grad_blocks(batch) x
+// (parameters + 1); grad: one set of parameters)
+int launch_train_steps(float* params, float* mstate, float* vstate, const float* X, const float* t,
+                       long long nsamples, int batch, long long per_epoch, long long mb0,
+                       int steps, const AdamStep* sched_host, AdamStep* sched, float* partials,
+                       float* grad, cudaStream_t s);
+// sums of squared residuals over the tiles of all minibatches, tile by tile
+// (train_loss_tiles values, at most one per sample)
+long long train_loss_tiles(long long nsamples, int batch);
+int launch_train_loss(const float* params, const float* X, const float* t, long long nsamples,
+                      int batch, float* out, cudaStream_t s);
+int mlp_train_configure();  // call once (returns != 0 on error)
 // where the network's outputs go: raw outputs (eps != NULL), or, in the
 // mapping, B of each worklist item's slot record
 struct InferSink {
