@@ -1013,7 +1013,7 @@ __device__ __noinline__ void fp64_collide(const F64Slots P, const CollideCoef<do
 // for the second, in slot order, took as much longer as the second gained.)
 
 // The uncovered cells of a tile are listed into the tile's stage in cell order
-// (r << 16 | x), hdr[0] = their number.  Lane k holds coverage word k of the
+// (r << 16 | x - the tile's first x), hdr[0] = their number.  Lane k holds coverage word k of the
 // tile, loaded a tile ahead; the words' places come from a warp scan, so the
 // rounds that write the entries of a word do not depend on one another.  (A
 // loop that carried the counts from word to word took 4.4 us for a tile of 256
@@ -1059,7 +1059,7 @@ __device__ __forceinline__ void list_uncovered(const LbmParams& P, const Tile& T
     const int r = T.nr == 1 ? 0 : (int)g.div_wpr.div((unsigned)lane);
     const int x0 = (T.xw + lane - r * g.wpr) * 32, n = g.nx - x0;
     u_l = (n >= 32 ? 0xffffffffu : (1u << (n > 0 ? n : 0)) - 1u) & ~m_l;
-    ent_l = (r << 16) | x0;
+    ent_l = (r << 16) | (x0 - 32 * T.xw);
   }
   const int cnt = __popc(u_l), incl = warp_scan(cnt, lane), first_l = incl - cnt;
   const unsigned below = (1u << lane) - 1u;
@@ -1253,7 +1253,7 @@ __global__ void __launch_bounds__(F64_THREADS, 1) lbm_fp64_kernel(LbmParams P) {
       const int i = ch * 32 + lane;
       bool act = i < L;
       const int le = ls[4 + (act ? i : L - 1)];
-      const int r = le >> 16, x = le & 0xffff;
+      const int r = le >> 16, x = 32 * tl.xw + (le & 0xffff);
       const int row = tl.row0 + r;
       const int z = (int)g.div_ny.div((unsigned)row);
       const int y = row - z * g.ny;
