@@ -1242,7 +1242,11 @@ __global__ void __launch_bounds__(F64_THREADS, 1) lbm_fp64_kernel(LbmParams P) {
     const int tile = (int)blockIdx.x + it * (int)gridDim.x;
     if (tile >= P.ntiles) break;
     const int s = it % S;
-    if (!mbar_wait(&full[s], (unsigned)(it / S) & 1u)) {
+    // first the end of the tile that had the stage before: a warp may be here
+    // before that tile was loaded, when full's phase before that still answers
+    // to the same parity
+    if ((it >= S && !mbar_wait(&empty[s], (unsigned)(it / S - 1) & 1u)) ||
+        !mbar_wait(&full[s], (unsigned)(it / S) & 1u)) {
       if (lane == 0) atomicOr(P.status, ST_TIMEOUT);
       break;
     }
@@ -1714,7 +1718,8 @@ int cell_prefetch_ahead(const Grid& g, int* ahead) {
 }
 
 // Tiles of the staged kernels: 256 cells (tile_rows rows) when the padded row
-// divides 256, else one row, in FP64 cut into segments of at most 8 words; as
+// divides 256, else one row (FP64: as many rows as 256 cells hold, longer rows
+// cut into segments of at most 8 words); as
 // many stages as fit the per-block budget (FP32: two blocks per SM; FP64: one
 // block, next to its forcing table and cell lists).  They serve FP64 and the
 // FP32 AA pattern; FP32 pull streaming runs faster on the one-cell-per-thread
@@ -1733,11 +1738,11 @@ int lbm_plan(const Grid& g, int prec, int aa, LbmPlan* plan) {
   const int optin = smem_optin();
   if (optin <= 0) return 1;
   const size_t esz = fp32 ? sizeof(float) : sizeof(double);
-  const int TR = (g.nxp <= 256 && 256 % g.nxp == 0) ? 256 / g.nxp : 1;
   // FP64: rows of more than 8 words in equal segments (each staged with two
   // cells more on either side); per stage the tile's cell list with a 16-byte
   // header
   const bool f64 = prec == PREC_FP64;
+  const int TR = g.nxp <= 256 && (f64 || 256 % g.nxp == 0) ? 256 / g.nxp : 1;
   const int nseg = f64 ? (g.wpr + 7) / 8 : 1;
   const int seg_words = (g.wpr + nseg - 1) / nseg;
   const int row_cells = nseg > 1 ? 32 * seg_words + 4 : g.nxp;
@@ -1752,6 +1757,14 @@ int lbm_plan(const Grid& g, int prec, int aa, LbmPlan* plan) {
   if (S < 2) {
     if (extra + 2 * (stage + list_stage) > (size_t)optin) return f64;
     S = 2;
+  }
+  // FP64: while a tile is not done, no ticket from S tiles later on is taken up,
+  // and the consumer warps hold two tickets each: they reach less than 2
+  // F64_CONSUMER_WARPS tickets further.  Those must end within S tiles more,
+  // for the waits on a stage's barriers to tell its phases apart.
+  if (f64) {
+    const int words = tile_cells / 32;
+    if ((2 * F64_CONSUMER_WARPS - 1 + words - 1) / words >= (int)S) return 1;
   }
   const size_t smem = extra + S * (stage + list_stage);
   const int w = g.wall[0] | (g.wall[1] << 1) | (g.wall[2] << 2);
