@@ -467,20 +467,19 @@ FX_FN int fx_top_velocity(int top, const double* V, int bits) {
   }
   return top;
 }
-constexpr int FX_VBITS_FULL = 2, FX_VBITS_MIXED = 3;
+constexpr int FX_VBITS_MIXED = 3;
 
 // Collision of one cell of a kind; put(q, value) takes the results.
 //  FX_FLUID  no particle.
-//  FX_FULL   one particle, B = 1, surface velocity V: the solid operator
-//            (Eq. 19) swaps each pair and adds the difference of the
-//            equilibria, d_q' = d_qbar + E_s(V) - E_s(U) + 3 w c.(V + U).
-//  FX_MIXED  one particle of weight B and surface velocity V (B = 0: none):
-//            d' = F + B (S - F), F the fluid collision and S the solid
-//            operator's result.  E is one above the cell's exponent (with
-//            |V| < 2^(E + 2)), so that twice S - F fits.
+//  FX_MIXED  one particle of weight B <= 1 and surface velocity V (B = 0:
+//            none): d' = F + B (S - F), F the fluid collision and S the solid
+//            operator's result (Eq. 19), which swaps each pair and adds the
+//            difference of the equilibria, d_q' = d_qbar + E_s(V) - E_s(U) +
+//            3 w c.(V + U).  E is one above the cell's exponent (with |V| <
+//            2^(E + 2)), so that twice S - F fits.
 // V: 4 values, surface velocity and weight.  force(Fc) takes the force
 // B (U - V - f) of Eq. 21.
-enum { FX_FLUID = 0, FX_MIXED = 1, FX_FULL = 2 };
+enum { FX_FLUID = 0, FX_MIXED = 1 };
 template <int KIND, typename Force, typename Put>
 FX_FN void fx_collide(const FxRates& c, const FxRow& row, int E, const double* d, const double* V,
                       Force force, Put put) {
@@ -489,14 +488,14 @@ FX_FN void fx_collide(const FxRates& c, const FxRow& row, int E, const double* d
   FxSolid M;
   FxCoef w{0, 0, 0, 0};
   fx_load(d, E, C);
-  const int o20 = (E - (KIND == FX_FULL ? FX_BITS : FX_BITS - 1)) * (1 << 20);
+  const int o20 = (E - (FX_BITS - 1)) * (1 << 20);
   const int dith = fx_dither(C.R);
-  if constexpr (KIND != FX_FULL) fx_fluid(c, row, E, C, dith, L);
-  if constexpr (KIND != FX_FLUID) {
+  fx_fluid(c, row, E, C, dith, L);
+  if constexpr (KIND == FX_MIXED) {
     const int n20 = (FX_BITS - E) << 20;
     double Fc[3];
     fx D[3], S[3];
-    if (KIND == FX_MIXED) w = fx_weight(V[3]);
+    w = fx_weight(V[3]);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       const fx v = dbl_to_fx(dbl_scale(V[i], n20));
@@ -504,9 +503,8 @@ FX_FN void fx_collide(const FxRates& c, const FxRow& row, int E, const double* d
       D[i] = fx_sub(v, U);
       S[i] = fx_add(v, U);
       // U - V - f
-      fx u = fx_sub(fx_sub(0, D[i]), fx_add(row.fh[i], row.fh[i]));
-      if (KIND == FX_MIXED) u = fx_mul(fx_add(u, u), w);
-      Fc[i] = fx_to_dbl(u, o20);
+      const fx u = fx_sub(fx_sub(0, D[i]), fx_add(row.fh[i], row.fh[i]));
+      Fc[i] = fx_to_dbl(fx_mul(fx_add(u, u), w), o20);
     }
     force(Fc);
     fx_solid(c, E, D, S, S, dith, M);
@@ -517,23 +515,15 @@ FX_FN void fx_collide(const FxRates& c, const FxRow& row, int E, const double* d
     return fx_add(F, fx_mul(fx_add(b, b), w));
   };
   if constexpr (KIND == FX_FLUID) put(0, fx_to_dbl(L.d0, o20));
-  else if constexpr (KIND == FX_FULL) put(0, fx_to_dbl(fx_add(C.x[0], M.d0), o20));
   else put(0, fx_to_dbl(blend(L.d0, fx_add(C.x[0], M.d0)), o20));
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
     fx qa, qb, sa, sb;
-    if constexpr (KIND != FX_FULL) fx_fluid_pair(c, row, C, L, k, &qa, &qb);
-    if constexpr (KIND != FX_FLUID) {
+    fx_fluid_pair(c, row, C, L, k, &qa, &qb);
+    if constexpr (KIND == FX_MIXED) {
       fx_solid_pair(M, k, &sa, &sb);
-      sa = fx_add(C.x[2 * k + 2], sa);
-      sb = fx_add(C.x[2 * k + 1], sb);
-    }
-    if constexpr (KIND == FX_FULL) {
-      qa = sa;
-      qb = sb;
-    } else if constexpr (KIND == FX_MIXED) {
-      qa = blend(qa, sa);
-      qb = blend(qb, sb);
+      qa = blend(qa, fx_add(C.x[2 * k + 2], sa));
+      qb = blend(qb, fx_add(C.x[2 * k + 1], sb));
     }
     put(2 * k + 1, fx_to_dbl(qa, o20));
     put(2 * k + 2, fx_to_dbl(qb, o20));

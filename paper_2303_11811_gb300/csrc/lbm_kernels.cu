@@ -809,7 +809,7 @@ __global__ void __launch_bounds__(BULK_THREADS, sizeof(T) == 4 ? 2 : 1)
 // ---- FP64 collision on compacted warps, for the cells that the fixed-point
 // form (fixed64.cuh) does not take: deviations or velocities of 1/8 and more,
 // NaN, cells of two particles.
-enum { CK_UNCOVERED = 0, CK_MIXED = 1, CK_FULL = 2 };
+enum { CK_UNCOVERED = 0, CK_MIXED = 1 };
 // consumer warps of the staged kernel: with the copy and the list warp a
 // multiple of four, which is what registers are shared out by.  14 (128
 // registers, no spills) measured best: 741 clocks of an SM per warp of cells
@@ -830,11 +830,6 @@ __device__ __forceinline__ void lds4(const double* p, double* o) {
 // S_k = (1 - omega+)/2 s_k + X_k, A_k = (1 - omega-)/2 a_k + Y_k,
 // X_k = (9/2 omega+ w c.U + G_k) c.U + C_c, Y_k = 3 omega- w c.U + F_k: seven
 // FP64 operations per pair instead of nine.
-// CK_FULL: every lane is a covered cell of one particle with B = 1; the fluid
-// change vanishes and the solid operator (Eq. 19) swaps the pair and adds the
-// difference of the equilibria: d_q' = d_qbar + (BdS + 3 w (cu + cv)),
-// d_qbar' = d_q + (BdS - 3 w (cu + cv)), BdS = w (9/2 (cv^2 - cu^2) -
-// 3/2 (V^2 - U^2)).
 // CK_MIXED: a covered lane (cov, slot index e) reads its slot records,
 // weights the fluid change by 1 - B and adds the solid operator of each of
 // its slots (Eq. 19); an uncovered lane has B = 0.
@@ -898,26 +893,6 @@ __device__ __noinline__ void fp64_collide(const F64Slots P, const CollideCoef<do
       d[2 * k + 1] = Sk + Ak;
       d[2 * k + 2] = Sk - Ak;
     }
-  } else if constexpr (KIND == CK_FULL) {
-    T r0[4] = {T(0), T(0), T(0), T(0)};
-    if (cov) ld4(P.V + 4LL * e, r0);
-    const T Vx = r0[0], Vy = r0[1], Vz = r0[2];
-    const T dU2 = (Vx * Vx + Vy * Vy + Vz * Vz) - uu;
-    d[0] += (T(-1.5) * w0<T>()) * dU2;
-    const T cd[2] = {(T(-1.5) * wk<T>(0)) * dU2, (T(-1.5) * wk<T>(3)) * dU2};
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      const int cl = k < 3 ? 0 : 1;
-      const T cu = cdot<T>(k, Ux, Uy, Uz);
-      const T cv = cdot<T>(k, Vx, Vy, Vz);
-      const T Sv = cv + cu;
-      const T BdS = (T(4.5) * wk<T>(cl == 0 ? 0 : 3)) * ((cv - cu) * Sv) + cd[cl];
-      const T t = (T(3) * wk<T>(cl == 0 ? 0 : 3)) * Sv;
-      const T dq = d[2 * k + 1];
-      d[2 * k + 1] = d[2 * k + 2] + (BdS + t);
-      d[2 * k + 2] = dq + (BdS - t);
-    }
-    if (cov) P.force(e, 0, T(1), Ux - Vx, Uy - Vy, Uz - Vz, h + CC_F);
   } else {
     // the cell's slots; the second one's record is read only when present
     T r0[4] = {T(0), T(0), T(0), T(0)}, r1[4] = {T(0), T(0), T(0), T(0)};
@@ -1004,13 +979,13 @@ __device__ __noinline__ void fp64_collide(const F64Slots P, const CollideCoef<do
 }
 
 // ---- the FP64 form's two kernels.  Cells without particles and covered cells
-// need code of 1,200 to 2,500 instructions each; run together, whether as
-// bodies of their own or as one with branches, they miss in the instruction
-// cache on a quarter of the cycles and more (settle512: 14.1 to 27 ms for the
-// collision).  So the uncovered cells have a kernel (staged rows), and the
-// covered cells, which the slot table lists in cell order, another that
-// gathers their 19 values.  (The first kernel copying them out of its stages
-// for the second, in slot order, took as much longer as the second gained.)
+// need code of 1,000 and 1,900 instructions; run together, whether as bodies of
+// their own or as one with branches, they miss in the instruction cache on a
+// quarter of the cycles and more (settle512: 14.1 to 27 ms for the collision).
+// So the uncovered cells have a kernel (staged rows), and the covered cells,
+// with the cells beside them, another that gathers their 19 values.  (The
+// first kernel copying them out of its stages for the second took as much
+// longer as the second gained.)
 
 // The uncovered cells of a tile are listed into the tile's stage in cell order
 // (r << 16 | x - the tile's first x), hdr[0] = their number.  Lane k holds coverage word k of the
@@ -1049,16 +1024,25 @@ __device__ __forceinline__ Tile tile_at(const LbmParams& P, int t, int nrows) {
   T.word0 = (size_t)T.row0 * g.wpr + T.xw;
   return T;
 }
+// Cells of the covered-cell kernel: those of the 4-cell groups (32-byte sectors
+// of a direction) with a covered cell in coverage word m.  With cells handed
+// over one by one, both kernels wrote parts of the sectors along the particles'
+// surfaces, and each part cost a read of its sector.
+__device__ __forceinline__ uint32_t covered_groups(uint32_t m) {
+  m |= m >> 2;
+  m = (m | (m >> 1)) & 0x11111111u;
+  return m * 15u;
+}
 // m_l: the lane's coverage word
 __device__ __forceinline__ void list_uncovered(const LbmParams& P, const Tile& T, uint32_t m_l,
                                                int* lst, int* hdr, int lane) {
   const Grid& g = P.g;
-  uint32_t u_l = 0u;  // uncovered live cells of the lane's word
+  uint32_t u_l = 0u;  // live cells of the lane's word outside covered groups
   int ent_l = 0;
   if (lane < T.words) {
     const int r = T.nr == 1 ? 0 : (int)g.div_wpr.div((unsigned)lane);
     const int x0 = (T.xw + lane - r * g.wpr) * 32, n = g.nx - x0;
-    u_l = (n >= 32 ? 0xffffffffu : (1u << (n > 0 ? n : 0)) - 1u) & ~m_l;
+    u_l = (n >= 32 ? 0xffffffffu : (1u << (n > 0 ? n : 0)) - 1u) & ~covered_groups(m_l);
     ent_l = (r << 16) | (x0 - 32 * T.xw);
   }
   const int cnt = __popc(u_l), incl = warp_scan(cnt, lane), first_l = incl - cnt;
@@ -1335,96 +1319,151 @@ __global__ void __launch_bounds__(F64_THREADS, 1) lbm_fp64_kernel(LbmParams P) {
   }
 }
 
-// Kernel of the covered cells: blocks claim groups of COV_GROUP slot entries
-// (consecutive covered cells), sort them by kind (one particle with B < 1, one
-// with B = 1, two particles) and take each kind's entries 32 at a time, so that
-// the block's warps run the same code at about the same time.  The cells of
-// two particles, few, run the FP64 form.  (Queues per warp, with the next 32
-// cells' values fetched by cp.async, let the kinds interleave in the
-// instruction cache and left each warp partly filled last chunks: 16% slower.)
-constexpr int COV_THREADS = 256, COV_GROUP = 1024;
-constexpr int COV_WARPS = COV_THREADS / 32, COV_ROUNDS = COV_GROUP / COV_THREADS;
+// Kernel of the covered cells and the rest of their 4-cell groups.  A block's
+// list warp claims spans of coverage words and lists the cells of COV_WORDS
+// words with particles at a time, seven consumer warps take them 32 at a time.
+// All cells of at most one particle run one body, the part form (B = 0 and 1
+// are exact in it): with bodies of their own for B = 1 and for uncovered cells
+// the warps missed in the instruction cache, and cells sorted by kind did not
+// share the lines they read and write.  The cells of two particles, few, are
+// listed from the end and run the FP64 form.
+// Collision of settle512, both kernels: 13.7 ms with a body per kind, barriers
+// and single cells; 12.1 with one body and 4-cell groups; 11.1 with the list
+// warp, which takes the barriers away and skips words without particles.  Now
+// DRAM traffic is 1.24 GB where it was 2.05 (256x256x128 settling box), warps
+// issue on 52% of the cycles, the FP64 pipe (conversions) is 54% busy.
+// Groups of 64 words measured 2% slower.  Copying the next 32 cells to shared
+// memory ahead did not help.
+constexpr int COV_THREADS = 256, COV_CONSUMER_WARPS = COV_THREADS / 32 - 1;
+constexpr int COV_WORDS = 128, COV_TURNS = 2;
+struct CovGroup {
+  unsigned short lst[32 * COV_WORDS];  // 32 word + cell in it
+  unsigned word[COV_WORDS];
+  uint32_t mask[COV_WORDS], two[COV_WORDS];
+  int base[COV_WORDS];
+  int one, twos;  // cells of at most one particle (-1: no group follows), of two
+  unsigned next;
+};
 template <int MODE, int WALLS>
 __global__ void __launch_bounds__(COV_THREADS, 2) lbm_fp64_covered_kernel(LbmParams P) {
   using T = double;
   const Grid& g = P.g;
   __shared__ FxRow rows[FX_ROWS];
-  __shared__ int2 lst[COV_GROUP];         // entry, padded cell
-  __shared__ int cnt[3][COV_GROUP / 32];  // per kind and 32 entries: count, then first place
-  __shared__ int tot[3];
-  __shared__ unsigned group, chunk;
+  __shared__ CovGroup groups[COV_TURNS];
+  __shared__ unsigned long long full[COV_TURNS], empty[COV_TURNS];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned all = 0xffffffffu, below = (1u << lane) - 1u;
-  const int n = (int)min((long long)*P.ncov, P.slot_cap);
   const F64Slots S{static_cast<const double*>(P.slot_V), static_cast<double*>(P.slot_Fc),
                    P.slot_cap};
   const int E0 = P.sc->fx_E0;
   for (int i = threadIdx.x; i < (int)(sizeof(rows) / sizeof(double2)); i += COV_THREADS)
     reinterpret_cast<double2*>(rows)[i] = reinterpret_cast<const double2*>(P.sc->fx)[i];
-  for (;;) {
-    __syncthreads();  // the previous group is done
-    if (threadIdx.x == 0) {
-      group = atomicAdd(P.work, 1u);
-      chunk = 0u;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < COV_TURNS; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], COV_CONSUMER_WARPS);
     }
-    __syncthreads();
-    const long long base = (long long)group * COV_GROUP;
-    if (base >= n) {
-      // each block ends on one claim too many: the last of them resets the
-      // counter for the next launch
-      const unsigned groups = (unsigned)((n + COV_GROUP - 1) / COV_GROUP);
-      if (threadIdx.x == 0 && group == groups + gridDim.x - 1) *P.work = 0u;
-      break;
-    }
-    // ---- kinds (2: B = 1, 1: two particles, 0: other) of the thread's entries
-    int kind[COV_ROUNDS], own[COV_ROUNDS];
-#pragma unroll
-    for (int j = 0; j < COV_ROUNDS; ++j) {
-      const long long e = base + j * COV_THREADS + threadIdx.x;
-      const double B = e < n ? S.V[4 * e + 3] : 0.0;
-      own[j] = e < n ? P.slot_cell[e] : 0;
-      kind[j] = e >= n ? -1 : (neg_flag(B) ? 1 : (B == 1.0 ? 2 : 0));
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const unsigned b = __ballot_sync(all, kind[j] == k);
-        if (lane == 0) cnt[k][j * COV_WARPS + warp] = __popc(b);
+  }
+  __syncthreads();
+  if (warp == COV_CONSUMER_WARPS) {
+    // ---- list warp
+    const unsigned nwords = (unsigned)g.nwords, span = (unsigned)P.cov_span;
+    const unsigned spans = (nwords + span - 1) / span;
+    auto claim = [&]() {
+      unsigned c = 0;
+      if (lane == 0) {
+        c = atomicAdd(P.work, 1u);
+        // each block ends on one claim too many: the last of them resets the
+        // counter for the next launch
+        if (c == spans + gridDim.x - 1) *P.work = 0u;
       }
-    }
-    __syncthreads();
-    if (warp < 3) {
-      static_assert(COV_GROUP / 32 == 32, "one lane per count");
-      const int v = cnt[warp][lane], incl = warp_scan(v, lane);
-      cnt[warp][lane] = incl - v;
-      if (lane == 31) tot[warp] = incl;
-    }
-    __syncthreads();
-    const int n0 = tot[0], n1 = tot[1], n2 = tot[2];
-#pragma unroll
-    for (int j = 0; j < COV_ROUNDS; ++j)
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const unsigned b = __ballot_sync(all, kind[j] == k);
-        if (kind[j] == k)
-          lst[(k == 0 ? 0 : (k == 1 ? n0 : n0 + n1)) + cnt[k][j * COV_WARPS + warp] +
-              __popc(b & below)] = make_int2(j * COV_THREADS + threadIdx.x, own[j]);
+      return __shfl_sync(all, c, 0);
+    };
+    // the next 32 words, their masks loaded one batch ahead
+    unsigned cur = claim(), w0 = cur * span, wend = min(w0 + span, nwords);
+    auto load = [&]() {
+      return cur < spans && w0 + lane < wend ? __ldg(&P.mask[w0 + lane]) : 0u;
+    };
+    uint32_t m = load();
+    for (int it = 0;; ++it) {
+      const int s = it % COV_TURNS;
+      if (it >= COV_TURNS && !mbar_wait(&empty[s], (unsigned)(it / COV_TURNS - 1) & 1u)) {
+        if (lane == 0) atomicOr(P.status, ST_TIMEOUT);
+        while (cur < spans) cur = claim();
+        break;
       }
-    __syncthreads();
-    const int c0 = (n0 + 31) / 32, c1 = (n1 + 31) / 32, c2 = (n2 + 31) / 32;
+      CovGroup& G = groups[s];
+      int count = 0;
+      while (cur < spans && count + 32 <= COV_WORDS) {
+        const unsigned b = __ballot_sync(all, m != 0u);
+        if (m) {
+          const int at = count + __popc(b & below);
+          G.word[at] = w0 + lane;
+          G.mask[at] = m;
+          G.two[at] = __ldg(&P.dup[w0 + lane]) & m;
+          G.base[at] = __ldg(&P.base[w0 + lane]);
+        }
+        count += __popc(b);
+        w0 += 32;
+        if (w0 >= wend) {
+          cur = claim();
+          w0 = cur * span;
+          wend = min(w0 + span, nwords);
+        }
+        m = load();
+      }
+      __syncwarp();
+      int one = 0, twos = 0;
+#pragma unroll 4
+      for (int v = 0; v < count; ++v) {
+        const unsigned wd = G.word[v], row = g.div_wpr.div(wd);
+        const int n = g.nx - (int)(wd - row * (unsigned)g.wpr) * 32;  // cells from here on
+        const uint32_t in = n >= 32 ? 0xffffffffu : (1u << n) - 1u;   // (not the row's padding)
+        const uint32_t t = G.two[v], o = covered_groups(G.mask[v]) & in & ~t;
+        const unsigned short ent = (unsigned short)(32 * v + lane);
+        if ((o >> lane) & 1u) G.lst[one + __popc(o & below)] = ent;
+        if ((t >> lane) & 1u) G.lst[32 * COV_WORDS - 1 - twos - __popc(t & below)] = ent;
+        one += __popc(o);
+        twos += __popc(t);
+      }
+      if (lane == 0) {
+        G.one = count > 0 ? one : -1;
+        G.twos = twos;
+        G.next = 0u;
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&full[s]);  // release: the lists are visible
+      if (count == 0) break;                 // no words are left
+    }
+    return;
+  }
+  // ---- consumers
+  for (int it = 0;; ++it) {
+    const int s = it % COV_TURNS;
+    if (!mbar_wait(&full[s], (unsigned)(it / COV_TURNS) & 1u)) {
+      if (lane == 0) atomicOr(P.status, ST_TIMEOUT);
+      return;
+    }
+    CovGroup& G = groups[s];
+    const int one = G.one, twos = G.twos;
+    if (one < 0) return;
+    const int c2 = (twos + 31) / 32, chunks = c2 + (one + 31) / 32;
     for (;;) {
       int c = 0;
-      if (lane == 0) c = (int)atomicAdd(&chunk, 1u);
+      if (lane == 0) c = (int)atomicAdd(&G.next, 1u);
       c = __shfl_sync(all, c, 0);
-      if (c >= c0 + c1 + c2) break;
-      // the longest first: two particles, mixed, full
-      const int kd = c < c1 ? 1 : (c < c1 + c0 ? 0 : 2);
-      const int first = kd == 0 ? 0 : (kd == 1 ? n0 : n0 + n1);
-      const int num = kd == 0 ? n0 : (kd == 1 ? n1 : n2);
-      const int i = 32 * (kd == 1 ? c : (kd == 0 ? c - c1 : c - c1 - c0)) + lane;
+      if (c >= chunks) break;
+      const bool two = c < c2;  // (the longest first)
+      const int i = 32 * (two ? c : c - c2) + lane, num = two ? twos : one;
       bool act = i < num;
-      const int2 le = lst[first + (act ? i : num - 1)];
-      const int e = (int)base + le.x, cell = le.y;
-      double V[4];
-      ld4(S.V + 4LL * e, V);
+      const int k = act ? i : num - 1;
+      const int li = G.lst[two ? 32 * COV_WORDS - 1 - k : k], lw = li >> 5;
+      const int cell = (int)(32u * G.word[lw]) + (li & 31);
+      const uint32_t m = G.mask[lw], bit = 1u << (li & 31);
+      const int e = G.base[lw] + __popc(m & (bit - 1u));
+      const bool covered = (m & bit) != 0u && e < P.slot_cap;
+      double V[4] = {0.0, 0.0, 0.0, 0.0};
+      if (covered) ld4(S.V + 4LL * e, V);
       const unsigned row = g.div_wpr.div((unsigned)cell >> 5);
       const int z = (int)g.div_ny.div(row);
       NbrT<WALLS> nb;
@@ -1451,17 +1490,16 @@ __global__ void __launch_bounds__(COV_THREADS, 2) lbm_fp64_covered_kernel(LbmPar
         if (act) store_pdf<T, MODE, WALLS>(P, nb, cell, q, v);
       };
       auto force = [&](const double* F) {
-        if (act) {
+        if (act && covered) {
           double* o = S.Fc + 3LL * e;
           o[0] = F[0];
           o[1] = F[1];
           o[2] = F[2];
         }
       };
-      int top = fx_top(d);
-      top = fx_top_velocity(top, V, kd == 2 ? FX_VBITS_FULL : FX_VBITS_MIXED);
-      FxRange R = fx_range(top, E0, kd == 2 ? 0 : 1, FX_EMAX_SOLID);
-      if (kd == 1) {
+      const int top = fx_top_velocity(fx_top(d), V, FX_VBITS_MIXED);
+      FxRange R = fx_range(top, E0, 1, FX_EMAX_SOLID);
+      if (two) {
         R.slow = true;
         R.quiet = false;
       }
@@ -1479,20 +1517,18 @@ __global__ void __launch_bounds__(COV_THREADS, 2) lbm_fp64_covered_kernel(LbmPar
         for (int q = 0; q < Q; ++q) t[q] = d[q];
         act = act && !R.slow;
       }
-      if (__any_sync(all, act) && E0 <= FX_EMAX_SOLID) {
-        const FxRow& row = rows[min(R.E - E0, FX_ROWS - 1)];
-        if (kd == 2) fx_collide<FX_FULL>(P.fx, row, R.E, d, V, force, put);
-        else fx_collide<FX_MIXED>(P.fx, row, R.E, d, V, force, put);
-      }
+      if (__any_sync(all, act) && E0 <= FX_EMAX_SOLID)
+        fx_collide<FX_MIXED>(P.fx, rows[min(R.E - E0, FX_ROWS - 1)], R.E, d, V, force, put);
       if (any_slow) {
-        const bool cov = live && R.slow;
-        if (kd == 2) fp64_collide<CK_FULL>(S, &P.sc->d, t, cov, cov ? e : -1);
-        else fp64_collide<CK_MIXED>(S, &P.sc->d, t, cov, cov ? e : -1);
-        act = cov;
+        act = live && R.slow;
+        const bool cov = act && covered;
+        fp64_collide<CK_MIXED>(S, &P.sc->d, t, cov, cov ? e : -1);
 #pragma unroll
         for (int q = 0; q < Q; ++q) put(q, t[q]);
       }
     }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&empty[s]);
   }
 #undef SRC
 }
@@ -1782,6 +1818,9 @@ int lbm_plan(const Grid& g, int prec, int aa, LbmPlan* plan) {
   plan->ntiles = (int)(nseg > 1 ? nrows * nseg : (nrows + TR - 1) / TR);
   plan->nseg = nseg;
   plan->cov_blocks = 2 * nsm;
+  // spans of at most 512 words, at least eight for each block of a large grid
+  const long long span = g.nwords / (8 * plan->cov_blocks) / 32 * 32;
+  plan->cov_span = (int)(span < 32 ? 32 : (span > 512 ? 512 : span));
   plan->seg_words = seg_words;
   plan->div_seg = make_fastdiv((unsigned)nseg);
   plan->stages = (int)S;
@@ -1795,9 +1834,9 @@ int lbm_plan(const Grid& g, int prec, int aa, LbmPlan* plan) {
 // The two kernels work on different cells (every value is read and written by
 // one cell only, in place or not), so they may run side by side.  They do where
 // the staged kernel has no more tiles than SMs and neither fills the device
-// (32^3: 20.1 us instead of 27.3); on larger grids the second kernel's blocks
-// keep the staged kernel's, one per SM, from starting (settle512: 15.5 ms
-// instead of 13.7).
+// (32^3: 18.0 us instead of 24.8); on larger grids the second kernel's blocks
+// keep the staged kernel's, one per SM, from starting (settle512: 12.1 ms
+// instead of 11.2).
 template <int MODE, int W>
 void launch_fp64(const LbmParams& P, size_t sm, const LbmFork& fk, cudaStream_t s) {
   if (!P.mask) {

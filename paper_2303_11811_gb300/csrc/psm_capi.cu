@@ -266,8 +266,7 @@ int enqueue_step(psm_ctx* c, bool with_map, cudaStream_t s, bool dem = true) {
   if (c->p.n > 0) {
     L.mask = c->cov.mask;
     L.base = c->cov.base;
-    L.ncov = c->cov.ncov;
-    L.slot_cell = c->slots.cell;
+    L.dup = c->cov.dup;
     L.work = c->work;
     L.slot_Fc = c->slots.Fc;
     L.slot_V = c->slots.V;
@@ -289,6 +288,7 @@ int enqueue_step(psm_ctx* c, bool with_map, cudaStream_t s, bool dem = true) {
   L.div_words = c->plan.div_words;
   L.div_seg = c->plan.div_seg;
   L.cov_blocks = c->plan.cov_blocks;
+  L.cov_span = c->plan.cov_span;
   L.pf_ahead = c->plan.pf_ahead;
   {
     NvtxRange r("psm stream-collide");

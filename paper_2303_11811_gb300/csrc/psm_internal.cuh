@@ -234,8 +234,7 @@ struct LbmParams {
   void* dstq[19];
   const uint32_t* mask; // nullptr when there are no particles
   const int* base;
-  const int* ncov;      // number of covered cells (Coverage::ncov)
-  const int* slot_cell; // Slots::cell
+  const uint32_t* dup;  // Coverage::dup
   unsigned* work;       // FP64: counter of the covered cells' groups
   void* slot_Fc;        // Slots::Fc
   const void* slot_V;   // Slots::V
@@ -255,6 +254,7 @@ struct LbmParams {
   int nseg, seg_words;
   FastDiv div_words, div_seg;
   int cov_blocks;       // blocks of the kernel of the covered cells
+  int cov_span;         // coverage words a block claims at a time
   // one-cell-per-thread FP32 pull kernel: each block prefetches into L2 the
   // source spans of the block pf_ahead places later (0: no prefetch)
   int pf_ahead;
@@ -266,6 +266,7 @@ struct LbmPlan {
   int nseg, seg_words;
   FastDiv div_words, div_seg;
   int cov_blocks;
+  int cov_span;
   int pf_ahead;
 };
 

@@ -61,8 +61,9 @@ static void collide(const double* din, double wp_, double wm_, const double* f_,
 static double rnd() { return 2.0 * drand48() - 1.0; }
 
 int main() {
-  const char* names[] = {"fluid", "mixed", "full"};
-  for (int kind = 0; kind < 3; ++kind)
+  // a covered cell of any weight, of weight 1, and none (B = 0), in the part form
+  const char* names[] = {"fluid", "mixed", "full", "none"};
+  for (int kind = 0; kind < 4; ++kind)
     for (double tau : {0.505, 0.55, 0.6, 1.0, 5.0})
       for (int trt = 0; trt < 2; ++trt)
         for (double um : {1e-12, 1e-5, 1e-3, 2e-2, 0.3})
@@ -76,8 +77,8 @@ int main() {
               for (int n = 0; n < 400; ++n) {
                 double f[3] = {fm * rnd(), fm * rnd(), fm * rnd()}, V[4], d[19];
                 for (int i = 0; i < 3; ++i) V[i] = um * rnd();
-                V[3] = kind == FX_FULL ? 1.0 : (n % 7 == 0 ? 0.0 : drand48());
-                if (kind == FX_FLUID) V[0] = V[1] = V[2] = V[3] = 0.0;
+                V[3] = kind == 2 ? 1.0 : (n % 7 == 0 ? 0.0 : drand48());
+                if (kind == FX_FLUID || kind == 3) V[0] = V[1] = V[2] = V[3] = 0.0;
                 if (wild) {  // any values below um, signs that add up in places
                   for (int q = 0; q < 19; ++q)
                     d[q] = um * (n % 3 == 0 ? (n % 2 ? 1.0 : -1.0) * (0.9 + 0.1 * drand48())
@@ -103,8 +104,8 @@ int main() {
                 const int E0 = fx_e0(c, f);
                 int top = fx_top(d);
                 if (kind != FX_FLUID)
-                  top = fx_top_velocity(top, V, kind == FX_FULL ? FX_VBITS_FULL : FX_VBITS_MIXED);
-                const int E = fx_exponent(top, E0) + (kind == FX_MIXED ? 1 : 0);
+                  top = fx_top_velocity(top, V, FX_VBITS_MIXED);
+                const int E = fx_exponent(top, E0) + (kind != FX_FLUID ? 1 : 0);
                 ++cells;
                 if (E > (kind == FX_FLUID ? FX_EMAX : FX_EMAX_SOLID)) {
                   ++out;
@@ -118,7 +119,6 @@ int main() {
                   for (int i = 0; i < 3; ++i) Fc[i] = F[i];
                 };
                 if (kind == FX_FLUID) fx_collide<FX_FLUID>(c, row, E, d, V, force, put);
-                else if (kind == FX_FULL) fx_collide<FX_FULL>(c, row, E, d, V, force, put);
                 else fx_collide<FX_MIXED>(c, row, E, d, V, force, put);
                 long double r[19], Fr[3];
                 double p[19], Fp[3];

@@ -39,7 +39,7 @@ def rows(tmp_path_factory):
     return r
 
 
-@pytest.mark.parametrize("kind", ["fluid", "mixed", "full"])
+@pytest.mark.parametrize("kind", ["fluid", "mixed", "full", "none"])
 def test_error_bound(rows, kind):
     """Every result within the unit bound, adversarial values included: a sum
     or product that overflowed would be off by orders of magnitude."""
@@ -61,7 +61,7 @@ def test_range(rows):
 def test_no_less_accurate_than_fp64(rows):
     """Near equilibrium, rms error over all settings of a kind, relative to the
     cell's largest value: at most that of FP64 arithmetic."""
-    for kind in ("fluid", "mixed", "full"):
+    for kind in ("fluid", "mixed", "full", "none"):
         sel = [r for r in rows if r["kind"] == kind and not r["wild"]
                and r["u"] in (1e-5, 1e-3, 2e-2) and r["f"] <= r["u"]]
         fixed = sum(r["rms"] ** 2 for r in sel) ** 0.5
