@@ -234,7 +234,6 @@ struct LbmParams {
   void* dstq[19];
   const uint32_t* mask; // nullptr when there are no particles
   const int* base;
-  const uint32_t* dup;  // Coverage::dup
   unsigned* work;       // FP64: counter of the covered cells' groups
   void* slot_Fc;        // Slots::Fc
   const void* slot_V;   // Slots::V
@@ -258,6 +257,10 @@ struct LbmParams {
   // one-cell-per-thread FP32 pull kernel: each block prefetches into L2 the
   // source spans of the block pf_ahead places later (0: no prefetch)
   int pf_ahead;
+  // FP64, covered cells: Coverage::dup (last: among the pointers above it moved
+  // the slots' to other 16-byte pairs, and the FP32 AA kernel's 96 registers did
+  // not suffice any more, 1.6% of its time)
+  const uint32_t* dup;
 };
 
 struct LbmPlan {
