@@ -34,7 +34,6 @@ constexpr int MAP_THREADS = 128;
 // 10 blocks per SM, 102 registers, 3% faster than 12 blocks at 85)
 constexpr int FILL_THREADS = 64;
 constexpr int FILL_MIN_BLOCKS = 10;
-constexpr int RED_THREADS = 128;
 constexpr int SCAN_THREADS = 1024;
 
 struct Box {
@@ -1501,40 +1500,33 @@ __global__ void vfluid_kernel(MapParams P, int nparts) {
 // values each lane carries at the first levels: 8 additions per lane instead
 // of 30.  Returns the total of value i in the lanes with (lane & 3) == 0 and
 // lane >> 2 = 4 (i / 3) + (i % 3) (lanes whose index maps to 3 or 7 carry an
-// empty slot).
-__device__ __forceinline__ double warp_sum6(const double (&v)[6], int lane, int& which) {
+// empty slot).  add(a, b): the sum of two values; from(v, o): lane ^ o's v.
+template <typename T, typename Add, typename From>
+__device__ __forceinline__ T warp_sum6(const T (&v)[6], T zero, int lane, int& which, Add add,
+                                       From from) {
   const bool b4 = (lane >> 4) & 1, b3 = (lane >> 3) & 1, b2 = (lane >> 2) & 1;
-  double w[4];
+  T w[4];
 #pragma unroll
-  for (int i = 0; i < 3; ++i) {  // lanes 0-15 keep values 0-2, lanes 16-31 values 3-5
-    const double keep = b4 ? v[i + 3] : v[i];
-    const double send = b4 ? v[i] : v[i + 3];
-    w[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-  }
-  w[3] = 0.0;
-  double u[2];
+  for (int i = 0; i < 3; ++i)  // lanes 0-15 keep values 0-2, lanes 16-31 values 3-5
+    w[i] = add(b4 ? v[i + 3] : v[i], from(b4 ? v[i] : v[i + 3], 16));
+  w[3] = zero;
+  T u[2];
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {  // then pairs {0,1} / {2,3}
-    const double keep = b3 ? w[i + 2] : w[i];
-    const double send = b3 ? w[i] : w[i + 2];
-    u[i] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-  }
-  {
-    const double keep = b2 ? u[1] : u[0];
-    const double send = b2 ? u[0] : u[1];
-    u[0] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-  }
-  u[0] += __shfl_xor_sync(0xffffffffu, u[0], 2);
-  u[0] += __shfl_xor_sync(0xffffffffu, u[0], 1);
+  for (int i = 0; i < 2; ++i)  // then pairs {0,1} / {2,3}
+    u[i] = add(b3 ? w[i + 2] : w[i], from(b3 ? w[i] : w[i + 2], 8));
+  u[0] = add(b2 ? u[1] : u[0], from(b2 ? u[0] : u[1], 4));
+  u[0] = add(u[0], from(u[0], 2));
+  u[0] = add(u[0], from(u[0], 1));
   const int j = 2 * b3 + b2;
   which = j < 3 ? 3 * b4 + j : -1;
   return u[0];
 }
 
 // A thread's walk over a particle's list entries k = threadIdx.x,
-// + RED_THREADS, ... with the list entries loaded two rounds ahead and the
+// + RT, ... with the list entries loaded two rounds ahead and the
 // next round's particle pair and cell one round ahead (the same entries in
 // the same order as a plain loop, so the sums are unchanged).
+template <int RT>
 struct ListWalk {
   const MapParams& P;
   long long loff;
@@ -1550,7 +1542,7 @@ struct ListWalk {
       pid1 = P.s.pid[e1];
       cell1 = P.s.cell[e1];
     }
-    if (k + RED_THREADS < cnt) e2 = P.list[loff + k + RED_THREADS];
+    if (k + RT < cnt) e2 = P.list[loff + k + RT];
   }
   // entry k's slot entry, particle pair and cell; loads ahead for k + 1, k + 2 rounds
   __device__ __forceinline__ void next(int k, int& e, int2& pid, int& cell) {
@@ -1558,17 +1550,25 @@ struct ListWalk {
     pid = pid1;
     cell = cell1;
     e1 = e2;
-    if (k + 2 * RED_THREADS < cnt) e2 = P.list[loff + k + 2 * RED_THREADS];
-    if (k + RED_THREADS < cnt) {
+    if (k + 2 * RT < cnt) e2 = P.list[loff + k + 2 * RT];
+    if (k + RT < cnt) {
       pid1 = P.s.pid[e1];
       cell1 = P.s.cell[e1];
     }
   }
 };
 
-template <typename T>
-__global__ void __launch_bounds__(RED_THREADS) force_reduce_kernel(MapParams P) {
-  __shared__ double sh[6][RED_THREADS / 32];
+// (double)k for |k| <= 2^24 without the FP64 pipe (a conversion takes 16 clocks
+// of it): the conversion to FP32 is exact, its bits move into place
+__device__ __forceinline__ double small_to_double(int k) {
+  const unsigned u = __float_as_uint((float)k);
+  const unsigned hi = (u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u);
+  return k == 0 ? 0.0 : __hiloint2double((int)hi, (int)(u << 29));
+}
+
+template <typename T, int RT>
+__global__ void __launch_bounds__(RT) force_reduce_kernel(MapParams P) {
+  __shared__ double sh[6][RT / 32];
   __shared__ int sip[3];
   __shared__ double sfr[3];
   const int p = blockIdx.x;
@@ -1583,10 +1583,12 @@ __global__ void __launch_bounds__(RED_THREADS) force_reduce_kernel(MapParams P) 
   }
   __syncthreads();
   const int dims[3] = {P.g.nx, P.g.ny, P.g.nz};
+  // a box offset is at most the grid's length
+  const bool small = max(dims[0], max(dims[1], dims[2])) <= 1 << 23;
   // F, then sum over cells of (k - i_p) x F_c
   double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-  ListWalk walk(P, loff, cnt);
-  for (int k = threadIdx.x; k < cnt; k += RED_THREADS) {
+  ListWalk<RT> walk(P, loff, cnt);
+  for (int k = threadIdx.x; k < cnt; k += RT) {
     int e, cell;
     int2 pid;
     walk.next(k, e, pid, cell);
@@ -1601,7 +1603,7 @@ __global__ void __launch_bounds__(RED_THREADS) force_reduce_kernel(MapParams P) 
         if (2 * k0 > dims[a]) k0 -= dims[a];
         else if (2 * k0 < -dims[a]) k0 += dims[a];
       }
-      kd[a] = (double)k0;
+      kd[a] = small ? small_to_double(k0) : (double)k0;
     }
     const long long fo = 3 * (s * P.s.cap + e);
     const double f0 = (double)Fc[fo];
@@ -1617,13 +1619,15 @@ __global__ void __launch_bounds__(RED_THREADS) force_reduce_kernel(MapParams P) 
   // fixed-order tree: within each warp by shuffles, then over the warps
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   int which;
-  const double ws = warp_sum6(acc, lane, which);
+  const double ws = warp_sum6(
+      acc, 0.0, lane, which, [](double a, double b) { return a + b; },
+      [](double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); });
   if ((lane & 3) == 0 && which >= 0) sh[which][wid] = ws;
   __syncthreads();
   if (threadIdx.x < 6) {
     const int i = threadIdx.x;
     double t = sh[i][0];
-    for (int w = 1; w < RED_THREADS / 32; ++w) t += sh[i][w];
+    for (int w = 1; w < RT / 32; ++w) t += sh[i][w];
     sh[i][0] = t;
   }
   __syncthreads();
@@ -1666,8 +1670,9 @@ struct FloatPair {
   __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
 
-__global__ void __launch_bounds__(RED_THREADS) force_reduce_f32_kernel(MapParams P) {
-  __shared__ FloatPair sh[6][RED_THREADS / 32];
+template <int RT>
+__global__ void __launch_bounds__(RT) force_reduce_f32_kernel(MapParams P) {
+  __shared__ FloatPair sh[6][RT / 32];
   __shared__ int sip[3];
   __shared__ float sfp[3];
   const int p = blockIdx.x;
@@ -1684,8 +1689,8 @@ __global__ void __launch_bounds__(RED_THREADS) force_reduce_f32_kernel(MapParams
   const int dims[3] = {P.g.nx, P.g.ny, P.g.nz};
   FloatPair acc[6];
   for (int i = 0; i < 6; ++i) acc[i] = FloatPair{0.f, 0.f};
-  ListWalk walk(P, loff, cnt);
-  for (int k = threadIdx.x; k < cnt; k += RED_THREADS) {
+  ListWalk<RT> walk(P, loff, cnt);
+  for (int k = threadIdx.x; k < cnt; k += RT) {
     int e, cell;
     int2 pid;
     walk.next(k, e, pid, cell);
@@ -1719,21 +1724,24 @@ __global__ void __launch_bounds__(RED_THREADS) force_reduce_f32_kernel(MapParams
   // fixed-order tree of the pairs: within each warp by shuffles, then over
   // the warps; one conversion to FP64 per component at the end
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int o = 16; o > 0; o >>= 1)
-    for (int i = 0; i < 6; ++i) {
-      FloatPair q;
-      q.hi = __shfl_down_sync(0xffffffffu, acc[i].hi, o);
-      q.lo = __shfl_down_sync(0xffffffffu, acc[i].lo, o);
-      acc[i].merge(q);
-    }
-  if (lane == 0)
-    for (int i = 0; i < 6; ++i) sh[i][wid] = acc[i];
+  int which;
+  const FloatPair ws = warp_sum6(
+      acc, FloatPair{0.f, 0.f}, lane, which,
+      [](FloatPair a, const FloatPair& b) {
+        a.merge(b);
+        return a;
+      },
+      [](const FloatPair& v, int o) {
+        return FloatPair{__shfl_xor_sync(0xffffffffu, v.hi, o),
+                         __shfl_xor_sync(0xffffffffu, v.lo, o)};
+      });
+  if ((lane & 3) == 0 && which >= 0) sh[which][wid] = ws;
   __syncthreads();
   if (threadIdx.x == 0) {
     double tot[6];
     for (int i = 0; i < 6; ++i) {
       FloatPair t = sh[i][0];
-      for (int w = 1; w < RED_THREADS / 32; ++w) t.merge(sh[i][w]);
+      for (int w = 1; w < RT / 32; ++w) t.merge(sh[i][w]);
       tot[i] = t.value();
     }
     bool finite = true;
@@ -1751,8 +1759,9 @@ __global__ void __launch_bounds__(RED_THREADS) force_reduce_f32_kernel(MapParams
 // centre) in double-float, products and sums in double-float on the FP32
 // pipes (df.cuh), the same fixed-order tree, one conversion to FP64 per
 // component at the end.
-__global__ void __launch_bounds__(RED_THREADS) force_reduce_df_kernel(MapParams P) {
-  __shared__ df sh[6][RED_THREADS / 32];
+template <int RT>
+__global__ void __launch_bounds__(RT) force_reduce_df_kernel(MapParams P) {
+  __shared__ df sh[6][RT / 32];
   __shared__ int sip[3];
   __shared__ df sfr[3];
   const int p = blockIdx.x;
@@ -1769,8 +1778,8 @@ __global__ void __launch_bounds__(RED_THREADS) force_reduce_df_kernel(MapParams 
   const int dims[3] = {P.g.nx, P.g.ny, P.g.nz};
   df acc[6];
   for (int i = 0; i < 6; ++i) acc[i] = df(0.f, 0.f);
-  ListWalk walk(P, loff, cnt);
-  for (int k = threadIdx.x; k < cnt; k += RED_THREADS) {
+  ListWalk<RT> walk(P, loff, cnt);
+  for (int k = threadIdx.x; k < cnt; k += RT) {
     int e, cell;
     int2 pid;
     walk.next(k, e, pid, cell);
@@ -1800,20 +1809,19 @@ __global__ void __launch_bounds__(RED_THREADS) force_reduce_df_kernel(MapParams 
     acc[5] = renorm(acc[5] + (d3[0] * f1 - d3[1] * f0));
   }
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int o = 16; o > 0; o >>= 1)
-    for (int i = 0; i < 6; ++i) {
-      const df q(__shfl_down_sync(0xffffffffu, acc[i].hi, o),
-                 __shfl_down_sync(0xffffffffu, acc[i].lo, o));
-      acc[i] = renorm(acc[i] + q);
-    }
-  if (lane == 0)
-    for (int i = 0; i < 6; ++i) sh[i][wid] = acc[i];
+  int which;
+  const df ws = warp_sum6(
+      acc, df(0.f, 0.f), lane, which, [](const df& a, const df& b) { return renorm(a + b); },
+      [](const df& v, int o) {
+        return df(__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o));
+      });
+  if ((lane & 3) == 0 && which >= 0) sh[which][wid] = ws;
   __syncthreads();
   if (threadIdx.x == 0) {
     double tot[6];
     for (int i = 0; i < 6; ++i) {
       df t = sh[i][0];
-      for (int w = 1; w < RED_THREADS / 32; ++w) t = renorm(t + sh[i][w]);
+      for (int w = 1; w < RT / 32; ++w) t = renorm(t + sh[i][w]);
       tot[i] = to_double(t);
     }
     bool finite = true;
@@ -1992,11 +2000,21 @@ int launch_weight_table(int n, double tau, int weighting, double* out, cudaStrea
   return 1;
 }
 
+template <int RT>
+void launch_force_reduce_t(const MapParams& P, cudaStream_t s) {
+  if (P.fp32) force_reduce_f32_kernel<RT><<<P.p.n, RT, 0, s>>>(P);
+  else if (P.dfrec) force_reduce_df_kernel<RT><<<P.p.n, RT, 0, s>>>(P);
+  else force_reduce_kernel<double, RT><<<P.p.n, RT, 0, s>>>(P);
+}
+
+// Blocks of 64 threads where the particles fill the device (fewer warps end on
+// a last round that is partly empty and on the sum over lanes: settle512 FP64
+// 882 -> 821 us, dense bed FP32 330 -> 302), of 128 where the latency of one
+// block counts (one sphere: 10.2 us, 13.8 with 64)
 int launch_force_reduce(MapParams P, cudaStream_t s) {
   if (P.p.n == 0) return 0;
-  if (P.fp32) force_reduce_f32_kernel<<<P.p.n, RED_THREADS, 0, s>>>(P);
-  else if (P.dfrec) force_reduce_df_kernel<<<P.p.n, RED_THREADS, 0, s>>>(P);
-  else force_reduce_kernel<double><<<P.p.n, RED_THREADS, 0, s>>>(P);
+  if (P.p.n >= 1024) launch_force_reduce_t<64>(P, s);
+  else launch_force_reduce_t<128>(P, s);
   return 1;
 }
 
