@@ -1832,44 +1832,27 @@ int lbm_plan(const Grid& g, int prec, int aa, LbmPlan* plan) {
 }
 
 // The two kernels work on different cells (every value is read and written by
-// one cell only, in place or not), so they may run side by side.  They do where
-// the staged kernel has no more tiles than SMs and neither fills the device
-// (32^3: 18.0 us instead of 24.8); on larger grids the second kernel's blocks
-// keep the staged kernel's, one per SM, from starting (settle512: 12.1 ms
-// instead of 11.2).
+// one cell only, in place or not) and run one after the other: side by side on
+// two streams they took settle512 from 11.2 to 12.1 ms (the second kernel's
+// blocks keep the staged kernel's, one per SM, from starting), and of the 7 us
+// they gained on 32^3 a replayed graph showed none.
 template <int MODE, int W>
-void launch_fp64(const LbmParams& P, size_t sm, const LbmFork& fk, cudaStream_t s) {
-  if (!P.mask) {
-    lbm_fp64_kernel<MODE, W><<<P.blocks, F64_THREADS, sm, s>>>(P);
-    return;
-  }
-  const bool beside = fk.side && P.ntiles <= P.blocks;
-  const cudaStream_t side = beside ? fk.side : s;
-  if (beside) {
-    cudaEventRecord(fk.fork, s);
-    cudaStreamWaitEvent(side, fk.fork, 0);
-  }
-  lbm_fp64_kernel<MODE, W><<<P.blocks, F64_THREADS, sm, s>>>(P);
-  lbm_fp64_covered_kernel<MODE, W><<<P.cov_blocks, COV_THREADS, 0, side>>>(P);
-  if (beside) {
-    cudaEventRecord(fk.join, side);
-    cudaStreamWaitEvent(s, fk.join, 0);
-  }
+void launch_fp64(const LbmParams& P, cudaStream_t s) {
+  lbm_fp64_kernel<MODE, W><<<P.blocks, F64_THREADS, P.smem, s>>>(P);
+  if (P.mask) lbm_fp64_covered_kernel<MODE, W><<<P.cov_blocks, COV_THREADS, 0, s>>>(P);
 }
 
 template <typename T, int W>
-void launch_lbm_t(const LbmParams& P, int mode, unsigned grid, const LbmFork& fk,
-                  cudaStream_t s) {
-  const size_t sm = P.smem;
+void launch_lbm_t(const LbmParams& P, int mode, unsigned grid, cudaStream_t s) {
   if constexpr (sizeof(T) == 8 && !kDF<T>) {
-    if (mode == 0) launch_fp64<0, W>(P, sm, fk, s);
-    else if (mode == 1) launch_fp64<1, W>(P, sm, fk, s);
-    else launch_fp64<2, W>(P, sm, fk, s);
+    if (mode == 0) launch_fp64<0, W>(P, s);
+    else if (mode == 1) launch_fp64<1, W>(P, s);
+    else launch_fp64<2, W>(P, s);
   } else {
     if constexpr (!kDF<T>) {  // plan.stages > 0: the AA pattern
       if (P.stages > 0) {
-        if (mode == 1) lbm_bulk_kernel<T, 1, W><<<P.blocks, BULK_THREADS, sm, s>>>(P);
-        else lbm_bulk_kernel<T, 2, W><<<P.blocks, BULK_THREADS, sm, s>>>(P);
+        if (mode == 1) lbm_bulk_kernel<T, 1, W><<<P.blocks, BULK_THREADS, P.smem, s>>>(P);
+        else lbm_bulk_kernel<T, 2, W><<<P.blocks, BULK_THREADS, P.smem, s>>>(P);
         return;
       }
     }
@@ -1880,15 +1863,14 @@ void launch_lbm_t(const LbmParams& P, int mode, unsigned grid, const LbmFork& fk
 }
 
 template <typename T>
-void launch_lbm_w(const LbmParams& P, int mode, unsigned grid, const LbmFork& fk,
-                  cudaStream_t s) {
+void launch_lbm_w(const LbmParams& P, int mode, unsigned grid, cudaStream_t s) {
   const int w = P.g.wall[0] | (P.g.wall[1] << 1) | (P.g.wall[2] << 2);
-  if (w == 0) launch_lbm_t<T, 0>(P, mode, grid, fk, s);
-  else if (w == 1) launch_lbm_t<T, 1>(P, mode, grid, fk, s);
-  else launch_lbm_t<T, 7>(P, mode, grid, fk, s);
+  if (w == 0) launch_lbm_t<T, 0>(P, mode, grid, s);
+  else if (w == 1) launch_lbm_t<T, 1>(P, mode, grid, s);
+  else launch_lbm_t<T, 7>(P, mode, grid, s);
 }
 
-int launch_lbm(const LbmParams& P0, int prec, int mode, const LbmFork& fk, cudaStream_t s) {
+int launch_lbm(const LbmParams& P0, int prec, int mode, cudaStream_t s) {
   LbmParams P = P0;
   const size_t esz = prec == PREC_FP32 ? sizeof(float) : sizeof(double);
   for (int q = 0; q < Q; ++q) {
@@ -1897,9 +1879,9 @@ int launch_lbm(const LbmParams& P0, int prec, int mode, const LbmFork& fk, cudaS
   }
   const long long threads = P.g.nwords * 32;
   const unsigned grid = (unsigned)((threads + LBM_THREADS - 1) / LBM_THREADS);
-  if (prec == PREC_FP32) launch_lbm_w<float>(P, mode, grid, fk, s);
-  else if (prec == PREC_DF) launch_lbm_w<df>(P, mode, grid, fk, s);
-  else launch_lbm_w<double>(P, mode, grid, fk, s);
+  if (prec == PREC_FP32) launch_lbm_w<float>(P, mode, grid, s);
+  else if (prec == PREC_DF) launch_lbm_w<df>(P, mode, grid, s);
+  else launch_lbm_w<double>(P, mode, grid, s);
   return prec == PREC_FP64 && P.mask ? 2 : 1;
 }
 

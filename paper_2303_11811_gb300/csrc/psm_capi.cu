@@ -44,7 +44,6 @@ struct psm_ctx {
   LbmPlan plan{};       // staged collision kernel (plan.stages = 0: not used)
   cudaStream_t stream = nullptr;
   cudaStream_t capture = nullptr;
-  LbmFork fork{};     // FP64: second stream of the collision
   std::vector<void*> allocs;
   void* buf[2] = {nullptr, nullptr};
   int cur = 0;        // pull: buffer holding f~ of the last step
@@ -292,7 +291,7 @@ int enqueue_step(psm_ctx* c, bool with_map, cudaStream_t s, bool dem = true) {
   L.pf_ahead = c->plan.pf_ahead;
   {
     NvtxRange r("psm stream-collide");
-    n += launch_lbm(L, c->prec, mode, c->fork, s);
+    n += launch_lbm(L, c->prec, mode, s);
   }
   if (c->timing) cudaEventRecord(c->ev[2], s);
   if (c->p.n > 0) {
@@ -626,13 +625,6 @@ psm_status psm_create(const psm_grid* grid, double tau, psm_relax relax, const p
   launch_step_const(map_params(c), s);
   c->have_wtab = launch_weight_table(c->opt.eps_n, c->tau, c->opt.weighting, c->wtab, s) > 0;
   if (cudaStreamCreateWithFlags(&c->capture, cudaStreamNonBlocking) != cudaSuccess) {
-    cudaGetLastError();
-    return bail(PSM_ERR_CUDA, "cudaStreamCreate failed");
-  }
-  if (c->prec == PREC_FP64 &&
-      (cudaStreamCreateWithFlags(&c->fork.side, cudaStreamNonBlocking) != cudaSuccess ||
-       cudaEventCreateWithFlags(&c->fork.fork, cudaEventDisableTiming) != cudaSuccess ||
-       cudaEventCreateWithFlags(&c->fork.join, cudaEventDisableTiming) != cudaSuccess)) {
     cudaGetLastError();
     return bail(PSM_ERR_CUDA, "cudaStreamCreate failed");
   }
@@ -1597,9 +1589,6 @@ void psm_destroy(psm_ctx* c) {
   for (auto& e : c->tev)
     if (e) cudaEventDestroy(e);
   if (c->capture) cudaStreamDestroy(c->capture);
-  if (c->fork.fork) cudaEventDestroy(c->fork.fork);
-  if (c->fork.join) cudaEventDestroy(c->fork.join);
-  if (c->fork.side) cudaStreamDestroy(c->fork.side);
   delete c;
 }
 

@@ -277,13 +277,7 @@ struct LbmPlan {
 int lbm_configure();  // kernel attributes; call once before launching (returns != 0 on error)
 // staged-kernel plan for a grid (stages = 0: use the one-cell-per-thread kernel)
 int lbm_plan(const Grid& g, int prec, int aa, LbmPlan* plan);
-// FP64: the covered cells' kernel runs beside the other on a second stream,
-// which forks from s and joins it again (side = nullptr: one after the other)
-struct LbmFork {
-  cudaStream_t side;
-  cudaEvent_t fork, join;
-};
-int launch_lbm(const LbmParams& P, int prec, int mode, const LbmFork& fk, cudaStream_t s);
+int launch_lbm(const LbmParams& P, int prec, int mode, cudaStream_t s);
 // a box of cells, origin (x0, y0, z0) (non-negative, taken modulo the grid) and
 // extent (bx, by, bz); output layout [q][z][y][x] over the box
 struct BoxSel {
