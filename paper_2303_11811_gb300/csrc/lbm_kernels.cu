@@ -807,8 +807,10 @@ __global__ void __launch_bounds__(BULK_THREADS, sizeof(T) == 4 ? 2 : 1)
 }
 
 // ---- FP64 collision on compacted warps, for the cells that the fixed-point
-// form (fixed64.cuh) does not take: deviations or velocities of 1/8 and more,
-// NaN, cells of two particles.
+// form (fixed64.cuh) does not take: a face direction's deviation of 1/8 and
+// more (beside a particle 1/32, for weights below 1/2 1/16) or the rest
+// direction's of 8 times that, a particle's velocity of 1/4 and more, NaN,
+// cells of two particles, and cells all but at rest under a force.
 enum { CK_UNCOVERED = 0, CK_MIXED = 1 };
 // consumer warps of the staged kernel: with the copy and the list warp a
 // multiple of four, which is what registers are shared out by.  14 (128
@@ -1057,20 +1059,17 @@ __device__ __forceinline__ void list_uncovered(const LbmParams& P, const Tile& T
   if (lane == 31) hdr[0] = incl;
 }
 
-// Range of the fixed-point form for a warp's cells: E of each lane; lanes
-// outside it (slow) go to the FP64 form, exactly quiescent cells without
-// forces get zeros (quiet)
-struct FxRange {
-  int E;
-  bool slow, quiet;
+// The forcing's constants of a cell's exponents (fixed64.cuh), from the block's
+// copy of the table
+struct RowsE {
+  const FxRow* rows;
+  int E0;
+  __device__ __forceinline__ const FxRow& operator()(int E) const {
+    return rows[min(E - E0, FX_ROWS - 1)];
+  }
 };
-__device__ __forceinline__ FxRange fx_range(int top, int E0, int add, int emax) {
-  FxRange r;
-  r.E = fx_exponent(top, E0) + add;
-  r.slow = r.E > emax;
-  r.quiet = E0 <= FX_EMIN && top == 0;
-  if (r.slow) r.E = E0;  // the lane's fixed-point result is not used
-  return r;
+__device__ __forceinline__ RowsE rows_p(const FxRow* rows, int E0) {
+  return RowsE{rows, fx_p0(E0)};
 }
 
 // Staged kernel of the cells without particles.  A copy warp streams each
@@ -1291,7 +1290,7 @@ __global__ void __launch_bounds__(F64_THREADS, 1) lbm_fp64_kernel(LbmParams P) {
       auto put = [&](int q, T v) {
         if (act) store_pdf<T, MODE, WALLS>(P, nb, cell, q, v);
       };
-      const FxRange R = fx_range(fx_top(d), E0, 0, FX_EMAX);
+      const FxRange R = fx_range<FX_FLUID>(d, nullptr, E0);
       if (R.quiet) {
 #pragma unroll
         for (int q = 0; q < Q; ++q) put(q, 0.0);
@@ -1304,9 +1303,9 @@ __global__ void __launch_bounds__(F64_THREADS, 1) lbm_fp64_kernel(LbmParams P) {
         for (int q = 0; q < Q; ++q) t[q] = d[q];
         act = act && !R.slow;
       }
-      if (__any_sync(0xffffffffu, act) && E0 <= FX_EMAX)
-        fx_collide<FX_FLUID>(P.fx, rows[min(R.E - E0, FX_ROWS - 1)], R.E, d, nullptr,
-                             [](const double*) {}, put);
+      if (__any_sync(0xffffffffu, act) && E0 <= FX_ETOP)
+        fx_cell<FX_FLUID>(P.fx, RowsE{rows, E0}, rows_p(rows, E0), E0, R.E, R.Ps, d, nullptr,
+                          [](const double*) {}, put);
       if (any_slow) {
         fp64_collide<CK_UNCOVERED>(F64Slots{nullptr, nullptr, 0}, &P.sc->d, t, false, -1);
         act = live && R.slow;
@@ -1497,8 +1496,7 @@ __global__ void __launch_bounds__(COV_THREADS, 2) lbm_fp64_covered_kernel(LbmPar
           o[2] = F[2];
         }
       };
-      const int top = fx_top_velocity(fx_top(d), V, FX_VBITS_MIXED);
-      FxRange R = fx_range(top, E0, 1, FX_EMAX_SOLID);
+      FxRange R = fx_range<FX_MIXED>(d, V, E0);
       if (two) {
         R.slow = true;
         R.quiet = false;
@@ -1517,8 +1515,9 @@ __global__ void __launch_bounds__(COV_THREADS, 2) lbm_fp64_covered_kernel(LbmPar
         for (int q = 0; q < Q; ++q) t[q] = d[q];
         act = act && !R.slow;
       }
-      if (__any_sync(all, act) && E0 <= FX_EMAX_SOLID)
-        fx_collide<FX_MIXED>(P.fx, rows[min(R.E - E0, FX_ROWS - 1)], R.E, d, V, force, put);
+      if (__any_sync(all, act) && E0 <= FX_ETOP)
+        fx_cell<FX_MIXED>(P.fx, RowsE{rows, E0}, rows_p(rows, E0), E0, R.E, R.Ps, d, V, force,
+                          put);
       if (any_slow) {
         act = live && R.slow;
         const bool cov = act && covered;
@@ -1978,7 +1977,8 @@ __global__ void __launch_bounds__(FX_ROWS) step_const_kernel(MapParams P) {
   if (P.fx_on) {
     const int E0 = fx_e0(P.fx, f);
     if (threadIdx.x == 0) sc->fx_E0 = E0;
-    if (E0 <= FX_EMAX) fx_row(P.fx, f, E0, threadIdx.x, sc->fx[threadIdx.x]);
+    if (E0 <= FX_ETOP)
+      fx_row_at(P.fx, f, E0 + threadIdx.x, fx_p0(E0) + threadIdx.x, sc->fx[threadIdx.x]);
   }
   if (threadIdx.x != 0) return;
   for (int a = 0; a < 3; ++a) sc->fext[a] = f[a];

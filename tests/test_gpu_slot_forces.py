@@ -1,0 +1,63 @@
+"""FP64 form: each covered cell's force B (U - V - f) (Eq. 21) after one step,
+where the density deviation is 2000 times the velocity and where the particle
+moves 100 times as fast as the fluid, against the same sum over the streamed
+deviations in extended precision.
+
+Bound, per component: FP64 holds the result to 2^-53 of itself and the
+collision's own error is a fraction of 2^-53 of the largest of |U|, |V|, |f|,
+times B: 2^-52 of that in all.
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+C = np.array([(0, 0, 0), (1, 0, 0), (-1, 0, 0), (0, 1, 0), (0, -1, 0), (0, 0, 1), (0, 0, -1),
+              (1, 1, 0), (-1, -1, 0), (1, -1, 0), (-1, 1, 0), (1, 0, 1), (-1, 0, -1), (1, 0, -1),
+              (-1, 0, 1), (0, 1, 1), (0, -1, -1), (0, 1, -1), (0, -1, 1)])
+W = np.array([1 / 3] + [1 / 18] * 6 + [1 / 36] * 12)
+
+
+@pytest.fixture(scope="module")
+def capi():
+    import torch
+    assert torch.cuda.is_available()
+    from paper_2303_11811_gb300 import build, capi as c
+    build.build()
+    return c
+
+
+@pytest.mark.parametrize("rho", [0.0, 2e-2, 0.3])
+@pytest.mark.parametrize("fbody", [(0.0, 0.0, 0.0), (1e-7, -3e-8, 2e-9)])
+def test_slot_forces(capi, rho, fbody):
+    n, um = 48, 1e-5
+    rng = np.random.default_rng(5)
+    u = um * (2.0 * rng.random((3, n, n, n)) - 1.0)
+    f = np.empty((19, n, n, n))
+    for q in range(19):
+        cu = np.tensordot(C[q], u, 1)
+        f[q] = W[q] * (1.0 + rho + 3.0 * cu + 4.5 * cu * cu - 1.5 * (u * u).sum(0))
+    x = np.array([[12.1, 12.4, 11.8], [34.3, 12.2, 30.9], [13.2, 35.4, 33.1]])
+    V = np.array([[0.0, 0.0, 0.0], [1e-3, -2e-3, 5e-4], [1e-5, 2e-5, -1e-5]])
+    e = capi.Engine(n, n, n, 0.55, relax="trt", fbody=fbody, weighting="nt",
+                    eps_mode="supersample", eps_n=8)
+    e.set_pdfs(f)
+    e.set_particles(x, np.array([5.3, 6.1, 4.2]), u=V, density=np.ones(3),
+                    fixed=np.ones(3, np.uint8))
+    e.step(1)
+    p0, B, p1, _ = e.slots()
+    _, _, F, _ = e.slot_forces()
+    assert (p1 < 0).all()
+    z, y, xx = np.nonzero(p0 >= 0)
+    j = np.zeros((z.size, 3), np.longdouble)
+    for q in range(1, 19):
+        d = f[q] - W[q]  # exact
+        j += d[(z - C[q][2]) % n, (y - C[q][1]) % n, (xx - C[q][0]) % n].astype(
+            np.longdouble)[:, None] * C[q]
+    B, F, v = B[z, y, xx], F[z, y, xx], V[p0[z, y, xx]]
+    fl = np.array(fbody, np.longdouble)
+    want = B[:, None] * (j - fl / 2 - v)
+    size = np.maximum(np.maximum(np.abs(j + fl / 2).max(1), np.abs(v).max(1)), np.abs(fl).max())
+    err = np.abs(F - want) / (2.0 ** -52 * B * size + (B == 0.0))[:, None]
+    assert (B > 0.0).sum() > 1000 and (B == 0.0).sum() > 100
+    assert err.max() <= 1.0
