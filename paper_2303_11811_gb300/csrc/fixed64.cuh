@@ -293,38 +293,54 @@ FX_FN int fx_e0(const FxRates& c, const double* f) {
   return e < FX_EMIN ? FX_EMIN : e;
 }
 
-// v 2^n rounded; *err gains w times the rounding error (in units)
+// v 2^n rounded, |n| < 1000; *err gains w times the rounding error (in units)
 FX_FN fx fx_round_err(double v, int n, double w, double* err) {
-  const double s = scalbn(v, n);  // exact
+  const double s = v * dbl_scale(1.0, n * (1 << 20));  // exact
   const fx y = dbl_to_fx(s);
   *err += w * ((double)y - s);
   return y;
 }
 
-// constants of the force density f (finite) for the exponents E and P
-FX_FN void fx_row_at(const FxRates& c, const double* f, int E, int P, FxRow& r) {
-  const double g = c.tau - 0.5, s2g = c.sigma[0] * c.sigma[0] * g * g;
-  const int out = FX_BITS - 1 - E;
-  for (int a = 0; a < 3; ++a) {
-    double none = 0.0, eg = 0.0;
-    r.fs[a] = fx_round_err(c.sigma[(E + 1) & 1] * c.tau * f[a], FX_BITS - E, 0.0, &none);
-    r.fh[a] = fx_round_err(0.5 * f[a], FX_BITS - E, 0.0, &none);
-    r.fg[a] = fx_round_err(f[a] / 6.0, out, 1.0, &eg);
-    // G enters a face pair once and its half the edge pairs twice net
-    r.compA[a] = (int)rint(-256.0 * (c.biasA[a] + 3.0 * eg));
-  }
-  const double ff = (f[0] * f[0] + f[1] * f[1] + f[2] * f[2]) / 3.0;
-  const double cf[6] = {f[0] + f[1], f[0] - f[1], f[0] + f[2],
-                        f[0] - f[2], f[1] + f[2], f[1] - f[2]};
-  double eF = 0.0, eD = 0.0, e0 = 0.0;
+// constants of the force density f (finite) for the exponents E and P, in
+// parts that the threads of step_const_kernel share: an axis, the face pairs
+// with the rest direction, the edge pairs
+FX_FN void fx_row_axis(const FxRates& c, double fa, int E, int a, FxRow& r) {
+  double none = 0.0, eg = 0.0;
+  r.fs[a] = fx_round_err(c.sigma[(E + 1) & 1] * c.tau * fa, FX_BITS - E, 0.0, &none);
+  r.fh[a] = fx_round_err(0.5 * fa, FX_BITS - E, 0.0, &none);
+  r.fg[a] = fx_round_err(fa / 6.0, FX_BITS - 1 - E, 1.0, &eg);
+  // G enters a face pair once and its half the edge pairs twice net
+  r.compA[a] = (int)rint(-256.0 * (c.biasA[a] + 3.0 * eg));
+}
+FX_FN double fx_s2g(const FxRates& c) {
+  const double g = c.tau - 0.5;
+  return c.sigma[0] * c.sigma[0] * g * g;
+}
+FX_FN double fx_third_of_square(const double* f) {
+  return (f[0] * f[0] + f[1] * f[1] + f[2] * f[2]) / 3.0;
+}
+FX_FN void fx_row_faces(const FxRates& c, const double* f, int E, int P, FxRow& r) {
+  const double s2g = fx_s2g(c), ff = fx_third_of_square(f);
+  double eF = 0.0, e0 = 0.0;
   for (int k = 0; k < 3; ++k)
-    r.K[k] = fx_round_err(2.0 * s2g * (ff - f[k] * f[k]), out, 1.0 / 3.0, &eF);
-  for (int k = 0; k < 6; ++k)
-    r.K[3 + k] = fx_round_err(s2g * (ff - cf[k] * cf[k]), out, 1.0 / 6.0, &eD);
+    r.K[k] = fx_round_err(2.0 * s2g * (ff - f[k] * f[k]), FX_BITS - 1 - E, 1.0 / 3.0, &eF);
   r.K0 = fx_round_err(12.0 * s2g * ff, FX_BITS - 1 - P, 1.0, &e0);
   r.compF = (int)rint(-256.0 * (c.biasS + eF));
-  r.compD = (int)rint(-256.0 * (c.biasS + eD));
   r.comp0 = (int)rint(-256.0 * (c.bias0 + e0));
+}
+FX_FN void fx_row_edges(const FxRates& c, const double* f, int E, FxRow& r) {
+  const double s2g = fx_s2g(c), ff = fx_third_of_square(f);
+  const double cf[6] = {f[0] + f[1], f[0] - f[1], f[0] + f[2],
+                        f[0] - f[2], f[1] + f[2], f[1] - f[2]};
+  double eD = 0.0;
+  for (int k = 0; k < 6; ++k)
+    r.K[3 + k] = fx_round_err(s2g * (ff - cf[k] * cf[k]), FX_BITS - 1 - E, 1.0 / 6.0, &eD);
+  r.compD = (int)rint(-256.0 * (c.biasS + eD));
+}
+FX_FN void fx_row_at(const FxRates& c, const double* f, int E, int P, FxRow& r) {
+  for (int a = 0; a < 3; ++a) fx_row_axis(c, f[a], E, a, r);
+  fx_row_faces(c, f, E, P, r);
+  fx_row_edges(c, f, E, r);
 }
 
 // half of x, rounded to the nearest integer, ties to even
