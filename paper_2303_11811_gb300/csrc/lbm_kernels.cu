@@ -1318,7 +1318,8 @@ __global__ void __launch_bounds__(F64_THREADS, 1) lbm_fp64_kernel(LbmParams P) {
   }
 }
 
-// Kernel of the covered cells and the rest of their 4-cell groups.  A block's
+// Kernel of the covered cells and the rest of their 4-cell groups (cov_all:
+// of every cell, B = 0 in most).  A block's
 // list warp claims spans of coverage words and lists the cells of COV_WORDS
 // words with particles at a time, seven consumer warps take them 32 at a time.
 // All cells of at most one particle run one body, the part form (B = 0 and 1
@@ -1335,6 +1336,8 @@ __global__ void __launch_bounds__(F64_THREADS, 1) lbm_fp64_kernel(LbmParams P) {
 // memory ahead did not help.
 constexpr int COV_THREADS = 256, COV_CONSUMER_WARPS = COV_THREADS / 32 - 1;
 constexpr int COV_WORDS = 128, COV_TURNS = 2;
+// chunks of 32 cells per consumer warp up to which this kernel runs alone (lbm_plan)
+constexpr int COV_ALL_CHUNKS = 8;
 struct CovGroup {
   unsigned short lst[32 * COV_WORDS];  // 32 word + cell in it
   unsigned word[COV_WORDS];
@@ -1368,8 +1371,13 @@ __global__ void __launch_bounds__(COV_THREADS, 2) lbm_fp64_covered_kernel(LbmPar
     // ---- list warp
     const unsigned nwords = (unsigned)g.nwords, span = (unsigned)P.cov_span;
     const unsigned spans = (nwords + span - 1) / span;
+    unsigned own = blockIdx.x;
     auto claim = [&]() {
-      unsigned c = 0;
+      unsigned c = own;
+      if (P.cov_all) {  // a span per block
+        own = spans;
+        return c;
+      }
       if (lane == 0) {
         c = atomicAdd(P.work, 1u);
         // each block ends on one claim too many: the last of them resets the
@@ -1394,8 +1402,9 @@ __global__ void __launch_bounds__(COV_THREADS, 2) lbm_fp64_covered_kernel(LbmPar
       CovGroup& G = groups[s];
       int count = 0;
       while (cur < spans && count + 32 <= COV_WORDS) {
-        const unsigned b = __ballot_sync(all, m != 0u);
-        if (m) {
+        const bool take = P.cov_all ? w0 + lane < wend : m != 0u;
+        const unsigned b = __ballot_sync(all, take);
+        if (take) {
           const int at = count + __popc(b & below);
           G.word[at] = w0 + lane;
           G.mask[at] = m;
@@ -1418,7 +1427,8 @@ __global__ void __launch_bounds__(COV_THREADS, 2) lbm_fp64_covered_kernel(LbmPar
         const unsigned wd = G.word[v], row = g.div_wpr.div(wd);
         const int n = g.nx - (int)(wd - row * (unsigned)g.wpr) * 32;  // cells from here on
         const uint32_t in = n >= 32 ? 0xffffffffu : (1u << n) - 1u;   // (not the row's padding)
-        const uint32_t t = G.two[v], o = covered_groups(G.mask[v]) & in & ~t;
+        const uint32_t t = G.two[v];
+        const uint32_t o = (P.cov_all ? in : covered_groups(G.mask[v]) & in) & ~t;
         const unsigned short ent = (unsigned short)(32 * v + lane);
         if ((o >> lane) & 1u) G.lst[one + __popc(o & below)] = ent;
         if ((t >> lane) & 1u) G.lst[32 * COV_WORDS - 1 - twos - __popc(t & below)] = ent;
@@ -1816,10 +1826,24 @@ int lbm_plan(const Grid& g, int prec, int aa, LbmPlan* plan) {
   plan->tile_rows = TR;
   plan->ntiles = (int)(nseg > 1 ? nrows * nseg : (nrows + TR - 1) / TR);
   plan->nseg = nseg;
-  plan->cov_blocks = 2 * nsm;
-  // spans of at most 512 words, at least eight for each block of a large grid
-  const long long span = g.nwords / (8 * plan->cov_blocks) / 32 * 32;
+  // spans of at most 512 words, at least eight for each block of a large grid;
+  // no more blocks than spans (a block copies the forcing table before it
+  // finds that nothing is left)
+  const long long span = g.nwords / (8 * 2 * nsm) / 32 * 32;
   plan->cov_span = (int)(span < 32 ? 32 : (span > 512 ? 512 : span));
+  const long long spans = (g.nwords + plan->cov_span - 1) / plan->cov_span;
+  plan->cov_blocks = (int)(spans < 2 * nsm ? spans : 2 * nsm);
+  // Small grids with particles: the covered-cell kernel takes every cell, a span
+  // of words per block.  Two kernels after one another cost such a step more
+  // than the bodies they save: a step of a drag measurement at 24^3 21.5 us
+  // against 32.6 (29.8 with one kernel of FP64 arithmetic), 32^3 27.8 / 38.1,
+  // 64^3 51.6 / 61.6, 70^3 (14,700 words) 67 / 79, 80^3 (19,200) 89 / 95, 96^3
+  // (27,648) 135 / 127, in place there 145 / 129.
+  if (g.nwords <= 2LL * nsm * COV_CONSUMER_WARPS * COV_ALL_CHUNKS) {
+    plan->cov_all = 1;
+    plan->cov_span = (int)((g.nwords + 2 * nsm - 1) / (2 * nsm));
+    plan->cov_blocks = (int)((g.nwords + plan->cov_span - 1) / plan->cov_span);
+  }
   plan->seg_words = seg_words;
   plan->div_seg = make_fastdiv((unsigned)nseg);
   plan->stages = (int)S;
@@ -1837,7 +1861,8 @@ int lbm_plan(const Grid& g, int prec, int aa, LbmPlan* plan) {
 // they gained on 32^3 a replayed graph showed none.
 template <int MODE, int W>
 void launch_fp64(const LbmParams& P, cudaStream_t s) {
-  lbm_fp64_kernel<MODE, W><<<P.blocks, F64_THREADS, P.smem, s>>>(P);
+  if (!P.mask || !P.cov_all)
+    lbm_fp64_kernel<MODE, W><<<P.blocks, F64_THREADS, P.smem, s>>>(P);
   if (P.mask) lbm_fp64_covered_kernel<MODE, W><<<P.cov_blocks, COV_THREADS, 0, s>>>(P);
 }
 
@@ -1881,7 +1906,7 @@ int launch_lbm(const LbmParams& P0, int prec, int mode, cudaStream_t s) {
   if (prec == PREC_FP32) launch_lbm_w<float>(P, mode, grid, s);
   else if (prec == PREC_DF) launch_lbm_w<df>(P, mode, grid, s);
   else launch_lbm_w<double>(P, mode, grid, s);
-  return prec == PREC_FP64 && P.mask ? 2 : 1;
+  return prec == PREC_FP64 && P.mask && !P.cov_all ? 2 : 1;
 }
 
 static unsigned grid_for(long long n, int block) {

@@ -288,6 +288,7 @@ int enqueue_step(psm_ctx* c, bool with_map, cudaStream_t s, bool dem = true) {
   L.div_seg = c->plan.div_seg;
   L.cov_blocks = c->plan.cov_blocks;
   L.cov_span = c->plan.cov_span;
+  L.cov_all = c->plan.cov_all;
   L.pf_ahead = c->plan.pf_ahead;
   {
     NvtxRange r("psm stream-collide");

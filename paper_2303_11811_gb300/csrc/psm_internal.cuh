@@ -254,6 +254,7 @@ struct LbmParams {
   FastDiv div_words, div_seg;
   int cov_blocks;       // blocks of the kernel of the covered cells
   int cov_span;         // coverage words a block claims at a time
+  int cov_all;          // that kernel takes every cell
   // one-cell-per-thread FP32 pull kernel: each block prefetches into L2 the
   // source spans of the block pf_ahead places later (0: no prefetch)
   int pf_ahead;
@@ -271,6 +272,7 @@ struct LbmPlan {
   FastDiv div_words, div_seg;
   int cov_blocks;
   int cov_span;
+  int cov_all;
   int pf_ahead;
 };
 
