@@ -655,8 +655,8 @@ __device__ __forceinline__ void bulk_copy_g2s(void* dst, const void* src, unsign
 }
 
 template <typename T, int MODE, int WALLS>
-__global__ void __launch_bounds__(BULK_THREADS, sizeof(T) == 4 ? 2 : 1)
-    lbm_bulk_kernel(LbmParams P) {
+__global__ void __launch_bounds__(BULK_THREADS, 2) lbm_bulk_kernel(LbmParams P) {
+  static_assert(sizeof(T) == 4 && MODE != 0, "FP32, in place");
   extern __shared__ __align__(128) unsigned char bulk_smem[];
   const Grid& g = P.g;
   unsigned long long* full = reinterpret_cast<unsigned long long*>(bulk_smem);
@@ -785,10 +785,7 @@ __global__ void __launch_bounds__(BULK_THREADS, sizeof(T) == 4 ? 2 : 1)
         const int qa = 2 * k + 1, qb = 2 * k + 2;
         const int xa = cx > 0 ? xm : (cx < 0 ? xq : x);  // x - c_x
         const int xb = cx > 0 ? xq : (cx < 0 ? xm : x);  // x + c_x
-        if (MODE == 0) {
-          d[qa] = nb.ok(-cx, -cy, -cz) ? sr[qa * C + xa] : ld(SRC(qb) + cell);
-          d[qb] = nb.ok(cx, cy, cz) ? sr[qb * C + xb] : ld(SRC(qa) + cell);
-        } else if (MODE == 1) {
+        if (MODE == 1) {
           d[qa] = sr[qa * C + x];
           d[qb] = sr[qb * C + x];
         } else {
@@ -796,7 +793,6 @@ __global__ void __launch_bounds__(BULK_THREADS, sizeof(T) == 4 ? 2 : 1)
           d[qb] = nb.ok(cx, cy, cz) ? sr[qb * C + xb] : ld(SRC(qb) + cell);
         }
       }
-      if constexpr (MODE == 0) apply_open_faces<T, WALLS>(P, nb, z, cell, d);
       psm_collide<T, true>(P, word, lane, live, d, m, eb, &R);
       if (live) store_pdfs<T, MODE, WALLS>(P, nb, cell, d);
     }
