@@ -160,20 +160,30 @@ class ClockSampler:
                 "samples": len(rows), "in_region": in_region}
 
 
-def source_hash(path):
-    with open(path, "rb") as f:
-        return hashlib.sha256(f.read()).hexdigest()[:16]
+def kernel_sources():
+    """The collision kernels' sources: the arithmetic of the FP64 and the
+    double-float form is in fixed64.cuh and df.cuh."""
+    csrc = os.path.join(ROOT, "paper_2303_11811_gb300", "csrc")
+    return [os.path.join(csrc, f) for f in ("lbm_kernels.cu", "fixed64.cuh", "df.cuh")]
 
 
-def profiled_traffic(kernel_src, name, cells):
-    """DRAM bytes per launch from the committed ncu summary, if the kernel
-    source is unchanged since the capture; else None.  A summary taken on a
+def source_hash(*paths):
+    h = hashlib.sha256()
+    for path in paths:
+        with open(path, "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
+
+
+def profiled_traffic(name, cells):
+    """DRAM bytes per launch from the committed ncu summary, if the kernel's
+    sources are unchanged since the capture; else None.  A summary taken on a
     smaller box of the same recipe gives bytes per cell
     (``dram_bytes_per_cell``), scaled here to `cells`."""
     path = os.path.join(ROOT, "profiles", f"{name}.md")
     if not os.path.exists(path):
         return None
-    want = source_hash(kernel_src)
+    want = source_hash(*kernel_sources())
     traffic, per_cell, h = None, None, None
     for line in open(path):
         if line.startswith("source_sha256_16:"):
@@ -616,9 +626,7 @@ def main():
         kbase = "lbm_bulk_kernel" if args.streaming == "aa" and args.precision == "fp32" \
             else "lbm_kernel"
         kname = kbase + f"<{ {'fp32': 'float', 'df64': 'df'}[args.precision] },{args.streaming}>"
-    traffic = profiled_traffic(os.path.join(ROOT, "paper_2303_11811_gb300", "csrc",
-                                            "lbm_kernels.cu"),
-                               f"{kbase}_{args.precision}{args.streaming}_{args.workload}", cells)
+    traffic = profiled_traffic(f"{kbase}_{args.precision}{args.streaming}_{args.workload}", cells)
     common = {"kernel": kname, "traffic": traffic, "covered_cells": ncov, "slots": nslot,
               "avg_launch_ms": lbm_ms,
               "class_ms_per_step": {"mapping": t[0] / t[4], "stream_collide": lbm_ms,
