@@ -85,7 +85,14 @@ typedef struct {
 
 typedef enum { PSM_SRT = 0, PSM_TRT = 1 } psm_relax;
 
-enum { PSM_FP64 = 0,       /* PDFs stored and collided in FP64 */
+enum { PSM_FP64 = 0,       /* PDFs stored as FP64 deviations f_q - w_q.  The
+                              collision runs in 64-bit block fixed point, with
+                              exponents per cell and kind of value and, on
+                              average over a class of results, no more rounding
+                              error than FP64 arithmetic; in FP64 arithmetic
+                              for cells of two particles and values outside its
+                              range (|f_q - w_q| from 1/8 on, beside particles
+                              1/32) */
        PSM_FP32_DEV = 1,   /* PDFs stored as FP32 deviations f_q - w_q,
                               collided in FP32; forces and checks in FP64 */
        PSM_FP64_DF = 2 };  /* PDFs stored as deviations in double-float form

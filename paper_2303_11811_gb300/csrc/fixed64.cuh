@@ -170,12 +170,11 @@ static_assert(sizeof(FxRow) % 16 == 0 && alignof(FxRow) == 16, "copied 16 bytes 
 constexpr int FX_ROWS = 64;
 FX_FN constexpr int fx_p0(int E0) { return 2 * E0 + 2; }
 // Directions whose conversion to an integer runs on the integer pipe, to
-// balance it against the FP64 pipe: 3 of 19 in cells without particles, 6 in
-// covered ones.  Collision of a 256^3 settling box 1.74 ms (1.77 with 3 and 3,
-// 1.79 with 12 and 3), of a channel at 20% solid fraction 1.03 (1.04, 1.08); a
-// box without particles takes 734 clocks of an SM per warp of cells with 3,
-// 751 with none, 719 with 12
-FX_FN constexpr bool fx_int_conv(int kind, int q) { return q < (kind ? 6 : 3); }
+// balance it against the FP64 pipe: 6 of 19.  Collision of a 256^3 settling box
+// 1.64 ms, of a channel at 20% solid fraction 0.98, of 256x128x128 without
+// particles 0.290 (none in cells without particles: 2% more, 2% less, 4% more;
+// 12 there: 2% and 2% more, 1% less)
+FX_FN constexpr bool fx_int_conv(int q) { return q < 6; }
 
 // FP64 words
 FX_FN int dbl_hi(double v) {
@@ -527,7 +526,7 @@ FX_FN void fx_cell(const FxRates& c, RowE rowE, RowP rowP, int E0, int E, int Ps
   constexpr int up = KIND == FX_MIXED ? 1 : 0;
   fx x[19], j[3], a[9], sf = 0, se = 0;
 #pragma unroll
-  for (int q = 1; q < 19; ++q) x[q] = fx_from(d[q], E, fx_int_conv(KIND, q));
+  for (int q = 1; q < 19; ++q) x[q] = fx_from(d[q], E, fx_int_conv(q));
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
     const fx s = fx_add(x[2 * k + 1], x[2 * k + 2]);
@@ -576,7 +575,7 @@ FX_FN void fx_cell(const FxRates& c, RowE rowE, RowP rowP, int E0, int E, int Ps
   }
   P += (P + E) & 1;
   const FxRow& rp = rowP(P);
-  const fx x0 = fx_from(d[0], P, fx_int_conv(KIND, 0));
+  const fx x0 = fx_from(d[0], P, fx_int_conv(0));
   const FxShift up_p = fx_shift(P - E, bits);
   const fx R = fx_add(x0, fx_add(fx_moved(sf, up_p), fx_moved(se, up_p)));
   FxFluid L;

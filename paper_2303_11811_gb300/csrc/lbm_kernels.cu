@@ -170,10 +170,6 @@ __device__ __forceinline__ void ld4(const df* p, df* o) {
 template <typename T>
 __device__ __forceinline__ const CollideCoef<T>* coef_of(const StepConst* sc);
 template <>
-__device__ __forceinline__ const CollideCoef<double>* coef_of<double>(const StepConst* sc) {
-  return &sc->d;
-}
-template <>
 __device__ __forceinline__ const CollideCoef<float>* coef_of<float>(const StepConst* sc) {
   return &sc->f;
 }
@@ -810,8 +806,9 @@ __global__ void __launch_bounds__(BULK_THREADS, 2) lbm_bulk_kernel(LbmParams P) 
 enum { CK_UNCOVERED = 0, CK_MIXED = 1 };
 // consumer warps of the staged kernel: with the copy and the list warp a
 // multiple of four, which is what registers are shared out by.  14 (128
-// registers, no spills) measured best: 741 clocks of an SM per warp of cells
-// with 10, 645 with 14, 18 (96 registers) no faster on boxes with particles
+// registers, no spills) measured best (with one exponent per cell): 741 clocks
+// of an SM per warp of cells with 10, 645 with 14, 18 (96 registers) no faster
+// on boxes with particles
 constexpr int F64_CONSUMER_WARPS = 14;
 constexpr int F64_THREADS = 32 * (F64_CONSUMER_WARPS + 2);
 constexpr int F64_FX_BYTES = (int)((sizeof(FxRow) * FX_ROWS + 127) / 128 * 128);
@@ -823,15 +820,39 @@ __device__ __forceinline__ void lds4(const double* p, double* o) {
 }
 
 // FP64 collision of one cell (Eqs. 3-8 and 17-21).
-// CK_UNCOVERED: all lanes of the warp are uncovered (B = 0); a pair's update
+// CK_UNCOVERED: the cell has no particle (B = 0); a pair's update
 // is written as d_q' = S_k + A_k, d_qbar' = S_k - A_k with
 // S_k = (1 - omega+)/2 s_k + X_k, A_k = (1 - omega-)/2 a_k + Y_k,
 // X_k = (9/2 omega+ w c.U + G_k) c.U + C_c, Y_k = 3 omega- w c.U + F_k: seven
 // FP64 operations per pair instead of nine.
-// CK_MIXED: a covered lane (cov, slot index e) reads its slot records,
+// CK_MIXED: a covered cell (cov, slot index e) reads its slot records,
 // weights the fluid change by 1 - B and adds the solid operator of each of
-// its slots (Eq. 19); an uncovered lane has B = 0.
-// Covered lanes write their slots' forces (Eq. 21).
+// its slots (Eq. 19); an uncovered one has B = 0.
+// Covered cells write their slots' forces (Eq. 21).
+
+// streaming into one cell (Eq. 2 read backwards; halfway bounce-back at walls)
+template <int MODE, int WALLS>
+__device__ __forceinline__ void gather_cell(const LbmParams& P, const NbrT<WALLS>& nb, int cell,
+                                            double* d) {
+#define SRC(q) static_cast<const double*>(P.srcq[q])
+  d[0] = ld(SRC(0) + cell);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const int cx = ckx(k), cy = cky(k), cz = ckz(k);
+    const int qa = 2 * k + 1, qb = 2 * k + 2;
+    if (MODE == 0) {
+      d[qa] = nb.ok(-cx, -cy, -cz) ? ld(SRC(qa) + nb.idx(-cx, -cy, -cz)) : ld(SRC(qb) + cell);
+      d[qb] = nb.ok(cx, cy, cz) ? ld(SRC(qb) + nb.idx(cx, cy, cz)) : ld(SRC(qa) + cell);
+    } else if (MODE == 1) {
+      d[qa] = ld(SRC(qa) + cell);
+      d[qb] = ld(SRC(qb) + cell);
+    } else {
+      d[qa] = nb.ok(-cx, -cy, -cz) ? ld(SRC(qb) + nb.idx(-cx, -cy, -cz)) : ld(SRC(qa) + cell);
+      d[qb] = nb.ok(cx, cy, cz) ? ld(SRC(qa) + nb.idx(cx, cy, cz)) : ld(SRC(qb) + cell);
+    }
+  }
+#undef SRC
+}
 
 struct F64Slots {
   const double* V;  // Slots::V
@@ -845,10 +866,9 @@ struct F64Slots {
     o[2] = Bi * (duz - f[2]);
   }
 };
-// (out of line: the fixed-point form takes almost every warp)
 template <int KIND>
-__device__ __noinline__ void fp64_collide(const F64Slots P, const CollideCoef<double>* cf,
-                                          double* d, bool cov, int e) {
+__device__ __forceinline__ void fp64_collide(const F64Slots& P, const CollideCoef<double>* cf,
+                                             double* d, bool cov, int e) {
   using T = double;
   T a[9], sk[9];
 #pragma unroll
@@ -952,7 +972,7 @@ __device__ __noinline__ void fp64_collide(const F64Slots P, const CollideCoef<do
     }
     if (cov) P.force(e, 0, B0, Ux - Vx, Uy - Vy, Uz - Vz, h + CC_F);
     // slot 1 (a cell shared by two particles: rare), on its own
-    if (__any_sync(0xffffffffu, has1) && has1) {
+    if (has1) {
       const T Wx = r1[0], Wy = r1[1], Wz = r1[2], B1 = r1[3];
       const T eU2 = (Wx * Wx + Wy * Wy + Wz * Wz) - uu;
       const T BeU = B1 * eU2;
@@ -976,21 +996,70 @@ __device__ __noinline__ void fp64_collide(const F64Slots P, const CollideCoef<do
   }
 }
 
+template <int WALLS>
+__device__ __forceinline__ int neighbours_of(const Grid& g, int cell, NbrT<WALLS>& nb) {
+  const unsigned row = g.div_wpr.div((unsigned)cell >> 5);
+  const int z = (int)g.div_ny.div(row);
+  nb.init(cell - (int)row * g.nxp, (int)row - z * g.ny, z, g.nx, g.ny, g.nz, g.nxp, g.wall);
+  return z;
+}
+
+// Stream and collide of one cell in FP64 arithmetic, for the lanes of either
+// kernel that the fixed-point form does not take.  Out of line and on its own,
+// from loading the cell's 19 values to storing them: with the values handed
+// over from the kernel's body and stored there, the copy and the second set of
+// stores cost the collision of a 256^3 settling box 5% (1.74 ms, 1.65 so), of a
+// channel 6%, of a box without particles 4%.  In place too: a cell's 19 values
+// are read and written by that cell alone.
+template <int KIND, int MODE, int WALLS>
+__device__ __noinline__ void fp64_cell(const LbmParams& P, int cell, bool cov, int e) {
+  using T = double;
+  NbrT<WALLS> nb;
+  const int z = neighbours_of<WALLS>(P.g, cell, nb);
+  T d[Q];
+  gather_cell<MODE, WALLS>(P, nb, cell, d);
+  if constexpr (MODE == 0) apply_open_faces<T, WALLS>(P, nb, z, cell, d);
+  const F64Slots S{static_cast<const double*>(P.slot_V), static_cast<double*>(P.slot_Fc),
+                   P.slot_cap};
+  fp64_collide<KIND>(S, &P.sc->d, d, cov, e);
+  store_pdfs<T, MODE, WALLS>(P, nb, cell, d);
+}
+// A quiescent cell without forces stays at rest (Fc: the force of its slot, or
+// nullptr).  Out of line as well: a set of stores more, or a loop of them, in
+// the kernels' bodies cost 2 to 3%.  (Pull and AA even write the cell's own
+// places, by plain addresses: the pointers of P would be loaded one by one here.)
+template <int MODE, int WALLS>
+__device__ __noinline__ void zero_cell(const LbmParams& P, double* dst, long long ncell, int cell,
+                                       double* Fc) {
+  if constexpr (MODE == 2) {
+    NbrT<WALLS> nb;
+    neighbours_of<WALLS>(P.g, cell, nb);
+    const double d[Q] = {};
+    store_pdfs<double, MODE, WALLS>(P, nb, cell, d);
+  } else {
+#pragma unroll
+    for (int q = 0; q < Q; ++q) dst[q * ncell + cell] = 0.0;
+  }
+  if (Fc) Fc[0] = Fc[1] = Fc[2] = 0.0;
+}
+
 // ---- the FP64 form's two kernels.  Cells without particles and covered cells
-// need code of 1,000 and 1,900 instructions; run together, whether as bodies of
-// their own or as one with branches, they miss in the instruction cache on a
-// quarter of the cycles and more (settle512: 14.1 to 27 ms for the collision).
+// need code of some 1,050 and 2,100 instructions; run together, whether as
+// bodies of their own or as one with branches, they miss in the instruction
+// cache on a quarter of the cycles and more (14.1 to 27 ms for the collision of
+// a 512^3 settling box, with one exponent per cell, that took 13.7 in two
+// kernels then).
 // So the uncovered cells have a kernel (staged rows), and the covered cells,
 // with the cells beside them, another that gathers their 19 values.  (The
 // first kernel copying them out of its stages for the second took as much
 // longer as the second gained.)
 
 // The uncovered cells of a tile are listed into the tile's stage in cell order
-// (r << 16 | x - the tile's first x), hdr[0] = their number.  Lane k holds coverage word k of the
-// tile, loaded a tile ahead; the words' places come from a warp scan, so the
-// rounds that write the entries of a word do not depend on one another.  (A
-// loop that carried the counts from word to word took 4.4 us for a tile of 256
-// cells and bound the kernel.)
+// (r << 16 | x - the tile's first x), hdr[0] = their number.  Lane k holds
+// coverage word k of the tile, loaded a tile ahead; the words' places come from
+// a warp scan, so the rounds that write the entries of a word do not depend on
+// one another.  (A loop that carried the counts from word to word took 4.4 us
+// for a tile of 256 cells and bound the kernel.)
 __device__ __forceinline__ int warp_scan(int v, int lane) {  // inclusive
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -1083,7 +1152,8 @@ __device__ __forceinline__ RowsE rows_p(const FxRow* rows, int E0) {
 // (Every warp visiting every tile cost a wait and a claim per warp and tile,
 // and left warps idle where a tile's chunks are not a multiple of them.)
 template <int MODE, int WALLS>
-__global__ void __launch_bounds__(F64_THREADS, 1) lbm_fp64_kernel(LbmParams P) {
+__global__ void __launch_bounds__(F64_THREADS, 1)
+    lbm_fp64_kernel(const __grid_constant__ LbmParams P) {
   using T = double;
   extern __shared__ __align__(128) unsigned char bulk_smem[];
   const Grid& g = P.g;
@@ -1107,7 +1177,8 @@ __global__ void __launch_bounds__(F64_THREADS, 1) lbm_fp64_kernel(LbmParams P) {
   {
     constexpr int NR = (int)(sizeof(FxRow) * FX_ROWS / sizeof(double2));
     const double2* srow = reinterpret_cast<const double2*>(P.sc->fx);
-    for (int i = threadIdx.x; i < NR; i += blockDim.x) reinterpret_cast<double2*>(rows)[i] = srow[i];
+    for (int i = threadIdx.x; i < NR; i += blockDim.x)
+      reinterpret_cast<double2*>(rows)[i] = srow[i];
   }
   if (threadIdx.x == 0) {
     *ticket = 0u;
@@ -1287,53 +1358,41 @@ __global__ void __launch_bounds__(F64_THREADS, 1) lbm_fp64_kernel(LbmParams P) {
         if (act) store_pdf<T, MODE, WALLS>(P, nb, cell, q, v);
       };
       const FxRange R = fx_range<FX_FLUID>(d, nullptr, E0);
-      if (R.quiet) {
-#pragma unroll
-        for (int q = 0; q < Q; ++q) put(q, 0.0);
-        act = false;
-      }
-      const bool live = act, any_slow = __any_sync(0xffffffffu, R.slow);
-      double t[Q];  // a copy: an array whose address is passed lives in memory
-      if (any_slow) {
-#pragma unroll
-        for (int q = 0; q < Q; ++q) t[q] = d[q];
-        act = act && !R.slow;
-      }
+      const bool quiet = act && R.quiet, slow = act && R.slow;
+      act = act && !R.quiet && !R.slow;
       if (__any_sync(0xffffffffu, act) && E0 <= FX_ETOP)
         fx_cell<FX_FLUID>(P.fx, RowsE{rows, E0}, rows_p(rows, E0), E0, R.E, R.Ps, d, nullptr,
                           [](const double*) {}, put);
-      if (any_slow) {
-        fp64_collide<CK_UNCOVERED>(F64Slots{nullptr, nullptr, 0}, &P.sc->d, t, false, -1);
-        act = live && R.slow;
-#pragma unroll
-        for (int q = 0; q < Q; ++q) put(q, t[q]);
-      }
+      if (quiet) zero_cell<MODE, WALLS>(P, static_cast<T*>(P.dst), g.ncell, cell, nullptr);
+      if (slow) fp64_cell<CK_UNCOVERED, MODE, WALLS>(P, cell, false, -1);
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(&empty[s]);
   }
 }
 
-// Kernel of the covered cells and the rest of their 4-cell groups (cov_all:
-// of every cell, B = 0 in most).  A block's
-// list warp claims spans of coverage words and lists the cells of COV_WORDS
-// words with particles at a time, seven consumer warps take them 32 at a time.
+// Kernel of the covered cells and the rest of their 4-cell groups (cov_all: of
+// every cell, B = 0 in most).  A block's list warp claims spans of coverage
+// words and lists the cells of COV_WORDS words with particles at a time, seven
+// consumer warps take them 32 at a time.
 // All cells of at most one particle run one body, the part form (B = 0 and 1
 // are exact in it): with bodies of their own for B = 1 and for uncovered cells
 // the warps missed in the instruction cache, and cells sorted by kind did not
 // share the lines they read and write.  The cells of two particles, few, are
 // listed from the end and run the FP64 form.
-// Collision of settle512, both kernels: 13.7 ms with a body per kind, barriers
-// and single cells; 12.1 with one body and 4-cell groups; 11.1 with the list
-// warp, which takes the barriers away and skips words without particles.  Now
-// DRAM traffic is 1.24 GB where it was 2.05 (256x256x128 settling box), warps
-// issue on 52% of the cycles, the FP64 pipe (conversions) is 54% busy.
-// Groups of 64 words measured 2% slower.  Copying the next 32 cells to shared
-// memory ahead did not help.
+// Collision of a 512^3 settling box, both kernels, with one exponent per cell:
+// 13.7 ms with a body per kind, barriers and single cells (DRAM traffic of a
+// 256x256x128 box 2.05 GB, 1.24 since); 12.1 with one body and 4-cell groups;
+// 11.1 with the list warp, which takes the barriers away and skips words
+// without particles.  With the exponents of fixed64.cuh 12.5: 11% more
+// instructions here, 6% in the staged kernel.  Warps issue on 47% of the
+// cycles, the FP64 pipe (conversions) is 53% busy, an eighth of the stalls are
+// instruction fetches.  Groups of 64 words measured 2% slower.  Copying the
+// next 32 cells to shared memory ahead did not help.
 constexpr int COV_THREADS = 256, COV_CONSUMER_WARPS = COV_THREADS / 32 - 1;
 constexpr int COV_WORDS = 128, COV_TURNS = 2;
 // chunks of 32 cells per consumer warp up to which this kernel runs alone (lbm_plan)
-constexpr int COV_ALL_CHUNKS = 8;
+constexpr int COV_ALL_CHUNKS = 10;
 struct CovGroup {
   unsigned short lst[32 * COV_WORDS];  // 32 word + cell in it
   unsigned word[COV_WORDS];
@@ -1343,7 +1402,8 @@ struct CovGroup {
   unsigned next;
 };
 template <int MODE, int WALLS>
-__global__ void __launch_bounds__(COV_THREADS, 2) lbm_fp64_covered_kernel(LbmParams P) {
+__global__ void __launch_bounds__(COV_THREADS, 2)
+    lbm_fp64_covered_kernel(const __grid_constant__ LbmParams P) {
   using T = double;
   const Grid& g = P.g;
   __shared__ FxRow rows[FX_ROWS];
@@ -1351,8 +1411,6 @@ __global__ void __launch_bounds__(COV_THREADS, 2) lbm_fp64_covered_kernel(LbmPar
   __shared__ unsigned long long full[COV_TURNS], empty[COV_TURNS];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned all = 0xffffffffu, below = (1u << lane) - 1u;
-  const F64Slots S{static_cast<const double*>(P.slot_V), static_cast<double*>(P.slot_Fc),
-                   P.slot_cap};
   const int E0 = P.sc->fx_E0;
   for (int i = threadIdx.x; i < (int)(sizeof(rows) / sizeof(double2)); i += COV_THREADS)
     reinterpret_cast<double2*>(rows)[i] = reinterpret_cast<const double2*>(P.sc->fx)[i];
@@ -1467,70 +1525,38 @@ __global__ void __launch_bounds__(COV_THREADS, 2) lbm_fp64_covered_kernel(LbmPar
       const uint32_t m = G.mask[lw], bit = 1u << (li & 31);
       const int e = G.base[lw] + __popc(m & (bit - 1u));
       const bool covered = (m & bit) != 0u && e < P.slot_cap;
-      double V[4] = {0.0, 0.0, 0.0, 0.0};
-      if (covered) ld4(S.V + 4LL * e, V);
-      const unsigned row = g.div_wpr.div((unsigned)cell >> 5);
-      const int z = (int)g.div_ny.div(row);
-      NbrT<WALLS> nb;
-      nb.init(cell - (int)row * g.nxp, (int)row - z * g.ny, z, g.nx, g.ny, g.nz, g.nxp, g.wall);
-      T d[Q];
-      d[0] = ld(SRC(0) + cell);
-#pragma unroll
-      for (int k = 0; k < 9; ++k) {
-        const int cx = ckx(k), cy = cky(k), cz = ckz(k);
-        const int qa = 2 * k + 1, qb = 2 * k + 2;
-        if (MODE == 0) {
-          d[qa] = nb.ok(-cx, -cy, -cz) ? ld(SRC(qa) + nb.idx(-cx, -cy, -cz)) : ld(SRC(qb) + cell);
-          d[qb] = nb.ok(cx, cy, cz) ? ld(SRC(qb) + nb.idx(cx, cy, cz)) : ld(SRC(qa) + cell);
-        } else if (MODE == 1) {
-          d[qa] = ld(SRC(qa) + cell);
-          d[qb] = ld(SRC(qb) + cell);
-        } else {
-          d[qa] = nb.ok(-cx, -cy, -cz) ? ld(SRC(qb) + nb.idx(-cx, -cy, -cz)) : ld(SRC(qa) + cell);
-          d[qb] = nb.ok(cx, cy, cz) ? ld(SRC(qa) + nb.idx(cx, cy, cz)) : ld(SRC(qb) + cell);
-        }
+      if (two) {
+        if (act) fp64_cell<CK_MIXED, MODE, WALLS>(P, cell, covered, e);
+        continue;
       }
+      double V[4] = {0.0, 0.0, 0.0, 0.0};
+      if (covered) ld4(static_cast<const double*>(P.slot_V) + 4LL * e, V);
+      NbrT<WALLS> nb;
+      const int z = neighbours_of<WALLS>(g, cell, nb);
+      T d[Q];
+      gather_cell<MODE, WALLS>(P, nb, cell, d);
       if constexpr (MODE == 0) apply_open_faces<T, WALLS>(P, nb, z, cell, d);
       auto put = [&](int q, T v) {
         if (act) store_pdf<T, MODE, WALLS>(P, nb, cell, q, v);
       };
       auto force = [&](const double* F) {
         if (act && covered) {
-          double* o = S.Fc + 3LL * e;
+          double* o = static_cast<double*>(P.slot_Fc) + 3LL * e;
           o[0] = F[0];
           o[1] = F[1];
           o[2] = F[2];
         }
       };
-      FxRange R = fx_range<FX_MIXED>(d, V, E0);
-      if (two) {
-        R.slow = true;
-        R.quiet = false;
-      }
-      if (R.quiet) {
-#pragma unroll
-        for (int q = 0; q < Q; ++q) put(q, 0.0);
-        const double zero[3] = {0.0, 0.0, 0.0};
-        force(zero);
-        act = false;
-      }
-      const bool live = act, any_slow = __any_sync(all, R.slow);
-      double t[Q];  // a copy: an array whose address is passed lives in memory
-      if (any_slow) {
-#pragma unroll
-        for (int q = 0; q < Q; ++q) t[q] = d[q];
-        act = act && !R.slow;
-      }
+      const FxRange R = fx_range<FX_MIXED>(d, V, E0);
+      const bool quiet = act && R.quiet, slow = act && R.slow;
+      act = act && !R.quiet && !R.slow;
       if (__any_sync(all, act) && E0 <= FX_ETOP)
         fx_cell<FX_MIXED>(P.fx, RowsE{rows, E0}, rows_p(rows, E0), E0, R.E, R.Ps, d, V, force,
                           put);
-      if (any_slow) {
-        act = live && R.slow;
-        const bool cov = act && covered;
-        fp64_collide<CK_MIXED>(S, &P.sc->d, t, cov, cov ? e : -1);
-#pragma unroll
-        for (int q = 0; q < Q; ++q) put(q, t[q]);
-      }
+      if (quiet)
+        zero_cell<MODE, WALLS>(P, static_cast<T*>(P.dst), g.ncell, cell,
+                               covered ? static_cast<double*>(P.slot_Fc) + 3LL * e : nullptr);
+      if (slow) fp64_cell<CK_MIXED, MODE, WALLS>(P, cell, covered, e);
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(&empty[s]);
@@ -1833,8 +1859,8 @@ int lbm_plan(const Grid& g, int prec, int aa, LbmPlan* plan) {
   // of words per block.  Two kernels after one another cost such a step more
   // than the bodies they save: a step of a drag measurement at 24^3 21.5 us
   // against 32.6 (29.8 with one kernel of FP64 arithmetic), 32^3 27.8 / 38.1,
-  // 64^3 51.6 / 61.6, 70^3 (14,700 words) 67 / 79, 80^3 (19,200) 89 / 95, 96^3
-  // (27,648) 135 / 127, in place there 145 / 129.
+  // 64^3 48.5 / 60.5, 70^3 (14,700 words) 65 / 77, 80^3 (19,200) 84 / 93, 96^3
+  // (27,648) 128 / 123, in place there 140 / 123.
   if (g.nwords <= 2LL * nsm * COV_CONSUMER_WARPS * COV_ALL_CHUNKS) {
     plan->cov_all = 1;
     plan->cov_span = (int)((g.nwords + 2 * nsm - 1) / (2 * nsm));
@@ -1852,9 +1878,9 @@ int lbm_plan(const Grid& g, int prec, int aa, LbmPlan* plan) {
 
 // The two kernels work on different cells (every value is read and written by
 // one cell only, in place or not) and run one after the other: side by side on
-// two streams they took settle512 from 11.2 to 12.1 ms (the second kernel's
-// blocks keep the staged kernel's, one per SM, from starting), and of the 7 us
-// they gained on 32^3 a replayed graph showed none.
+// two streams they took a 512^3 settling box from 11.2 to 12.1 ms (the second
+// kernel's blocks keep the staged kernel's, one per SM, from starting), and of
+// the 7 us they gained on 32^3 a replayed graph showed none.
 template <int MODE, int W>
 void launch_fp64(const LbmParams& P, cudaStream_t s) {
   if (!P.mask || !P.cov_all)
@@ -1993,8 +2019,9 @@ __device__ void fill_coef(CollideCoef<T>& c, const double* f, double wp, double 
 // Every step of moving particles waits for this kernel: a chain of FP64
 // operations, so its parts go to threads of their own, and a form fills its own
 // coefficients only: 5.7 us in the FP64 and the double-float form, 4.2 in FP32
-// (15.7, 12.2 and 6.9 with a thread for all coefficients and one per row).  Block 0: the coefficients; FP64 form: blocks 1 to 5 a part
-// each of the fixed-point collision's table, a thread per row.
+// (15.7, 12.2 and 6.9 with a thread for all coefficients and one per row).
+// Block 0: the coefficients; FP64 form: blocks 1 to 5 a part each of the
+// fixed-point collision's table, a thread per row.
 __global__ void __launch_bounds__(FX_ROWS) step_const_kernel(MapParams P) {
   StepConst* sc = P.sc;
   const double vf = sc->vfluid;

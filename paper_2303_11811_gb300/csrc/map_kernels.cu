@@ -2008,9 +2008,10 @@ void launch_force_reduce_t(const MapParams& P, cudaStream_t s) {
 }
 
 // Blocks of 64 threads where the particles fill the device (fewer warps end on
-// a last round that is partly empty and on the sum over lanes: settle512 FP64
-// 882 -> 821 us, dense bed FP32 330 -> 302), of 128 where the latency of one
-// block counts (one sphere: 10.2 us, 13.8 with 64)
+// a last round that is partly empty and on the sum over lanes: 512^3 settling
+// box FP64 882 -> 821 us, dense bed FP32 330 -> 302; of whole passes 1% and
+// less), of 128 where the latency of one block counts (one sphere: 10.2 us,
+// 13.8 with 64)
 int launch_force_reduce(MapParams P, cudaStream_t s) {
   if (P.p.n == 0) return 0;
   if (P.p.n >= 1024) launch_force_reduce_t<64>(P, s);
