@@ -1,7 +1,7 @@
 """FP64 form: each covered cell's force B (U - V - f) (Eq. 21) after one step,
-where the density deviation is 2000 times the velocity and where the particle
-moves 100 times as fast as the fluid, against the same sum over the streamed
-deviations in extended precision.
+at velocities of 1e-5 and 1e-12, where the density deviation is up to 30,000
+times the velocity and where the particle moves 100 times as fast as the fluid,
+against the same sum over the streamed deviations in extended precision.
 
 Bound, per component: FP64 holds the result to 2^-53 of itself and the
 collision's own error is a fraction of 2^-53 of the largest of |U|, |V|, |f|,
@@ -27,10 +27,12 @@ def capi():
     return c
 
 
-@pytest.mark.parametrize("rho", [0.0, 2e-2, 0.3])
-@pytest.mark.parametrize("fbody", [(0.0, 0.0, 0.0), (1e-7, -3e-8, 2e-9)])
-def test_slot_forces(capi, rho, fbody):
-    n, um = 48, 1e-5
+@pytest.mark.parametrize("um,rho", [(1e-5, 0.0), (1e-5, 2e-2), (1e-5, 0.3), (1e-12, 0.0),
+                                    (1e-12, 1e-8)])
+@pytest.mark.parametrize("f", [(0.0, 0.0, 0.0), (1e-2, -3e-3, 2e-4)])
+def test_slot_forces(capi, um, rho, f):
+    n = 48
+    fbody = tuple(um * v for v in f)
     rng = np.random.default_rng(5)
     u = um * (2.0 * rng.random((3, n, n, n)) - 1.0)
     f = np.empty((19, n, n, n))
@@ -38,7 +40,7 @@ def test_slot_forces(capi, rho, fbody):
         cu = np.tensordot(C[q], u, 1)
         f[q] = W[q] * (1.0 + rho + 3.0 * cu + 4.5 * cu * cu - 1.5 * (u * u).sum(0))
     x = np.array([[12.1, 12.4, 11.8], [34.3, 12.2, 30.9], [13.2, 35.4, 33.1]])
-    V = np.array([[0.0, 0.0, 0.0], [1e-3, -2e-3, 5e-4], [1e-5, 2e-5, -1e-5]])
+    V = um * np.array([[0.0, 0.0, 0.0], [100.0, -200.0, 50.0], [1.0, 2.0, -1.0]])
     e = capi.Engine(n, n, n, 0.55, relax="trt", fbody=fbody, weighting="nt",
                     eps_mode="supersample", eps_n=8)
     e.set_pdfs(f)
