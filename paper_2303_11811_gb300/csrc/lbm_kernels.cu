@@ -819,17 +819,6 @@ __device__ __forceinline__ void lds4(const double* p, double* o) {
   o[0] = u.x; o[1] = u.y; o[2] = v.x; o[3] = v.y;
 }
 
-// FP64 collision of one cell (Eqs. 3-8 and 17-21).
-// CK_UNCOVERED: the cell has no particle (B = 0); a pair's update
-// is written as d_q' = S_k + A_k, d_qbar' = S_k - A_k with
-// S_k = (1 - omega+)/2 s_k + X_k, A_k = (1 - omega-)/2 a_k + Y_k,
-// X_k = (9/2 omega+ w c.U + G_k) c.U + C_c, Y_k = 3 omega- w c.U + F_k: seven
-// FP64 operations per pair instead of nine.
-// CK_MIXED: a covered cell (cov, slot index e) reads its slot records,
-// weights the fluid change by 1 - B and adds the solid operator of each of
-// its slots (Eq. 19); an uncovered one has B = 0.
-// Covered cells write their slots' forces (Eq. 21).
-
 // streaming into one cell (Eq. 2 read backwards; halfway bounce-back at walls)
 template <int MODE, int WALLS>
 __device__ __forceinline__ void gather_cell(const LbmParams& P, const NbrT<WALLS>& nb, int cell,
@@ -866,6 +855,16 @@ struct F64Slots {
     o[2] = Bi * (duz - f[2]);
   }
 };
+// FP64 collision of one cell (Eqs. 3-8 and 17-21).
+// CK_UNCOVERED: the cell has no particle (B = 0); a pair's update
+// is written as d_q' = S_k + A_k, d_qbar' = S_k - A_k with
+// S_k = (1 - omega+)/2 s_k + X_k, A_k = (1 - omega-)/2 a_k + Y_k,
+// X_k = (9/2 omega+ w c.U + G_k) c.U + C_c, Y_k = 3 omega- w c.U + F_k: seven
+// FP64 operations per pair instead of nine.
+// CK_MIXED: a covered cell (cov, slot index e) reads its slot records,
+// weights the fluid change by 1 - B and adds the solid operator of each of
+// its slots (Eq. 19); an uncovered one has B = 0.
+// Covered cells write their slots' forces (Eq. 21).
 template <int KIND>
 __device__ __forceinline__ void fp64_collide(const F64Slots& P, const CollideCoef<double>* cf,
                                              double* d, bool cov, int e) {
